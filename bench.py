@@ -38,7 +38,8 @@ BYTES_PER_RAY_RENDER = 12 + 4                          # rgb + count written
 # Sources the dominant kernel (march_fwd_kernel<float, sparse, render>) is
 # compiled from: a recorded DRAM traffic figure is valid only for the sources
 # it was captured with.
-RENDER_SOURCES = ("paper_2404_09531_gb300/csrc/march_fwd.cu", "paper_2404_09531_gb300/csrc/packed.cuh",
+RENDER_SOURCES = ("paper_2404_09531_gb300/csrc/march_cam.cu", "paper_2404_09531_gb300/csrc/march_fwd.cu",
+                  "paper_2404_09531_gb300/csrc/march_fwd.cuh", "paper_2404_09531_gb300/csrc/packed.cuh",
                   "paper_2404_09531_gb300/csrc/common.cuh", "paper_2404_09531_gb300/csrc/mlp_mma.cuh")
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of that kernel
 # over the step's eight 1920x1080 cameras (one ncu capture), with the hash of

@@ -158,6 +158,28 @@ __device__ __forceinline__ bool lattice_test(const Geo& g, const float o[3], con
   return zb.x < p[2] && p[2] < zb.y;
 }
 
+// lattice_test for a caller that keeps the last cell it read and that cell's
+// interval: neighbouring samples of a ray mostly fall into one cell.
+__device__ __forceinline__ bool lattice_test_cached(const Geo& g, const float o[3], const float d[3], int k,
+                                                    float p[3], float2& zb, int& cell) {
+  float t = __fmul_rn((float)k, g.step);
+#pragma unroll
+  for (int a = 0; a < 3; a++) p[a] = __fadd_rn(o[a], __fmul_rn(t, d[a]));
+  if (!(p[0] >= g.lo[0] && p[0] <= g.hi[0] && p[1] >= g.lo[1] && p[1] <= g.hi[1] && p[2] >= g.lo[2] &&
+        p[2] <= g.hi[2]))
+    return false;
+  int cx = (int)floorf(__fmul_rn(__fsub_rn(p[0], g.lo[0]), g.osx));
+  int cy = (int)floorf(__fmul_rn(__fsub_rn(p[1], g.lo[1]), g.osy));
+  cx = min(max(cx, 0), g.M - 1);
+  cy = min(max(cy, 0), g.M - 1);
+  const int c = cx * g.M + cy;
+  if (c != cell) {
+    cell = c;
+    zb = __ldg(g.occ + c);
+  }
+  return zb.x < p[2] && p[2] < zb.y;
+}
+
 // Empty-space skipping (Sec. 4.4: max-pooled occupancy planes and box tests).
 // Lane j reports whether lattice window [kb + 32 j, kb + 32 j + 31] (clipped
 // to kh) may hold an evaluated sample: the window's sample positions lie in
@@ -167,48 +189,48 @@ __device__ __forceinline__ bool lattice_test(const Geo& g, const float o[3], con
 // sample can pass only if its z meets the max-pooled interval of a coarse
 // cell in that range.  Windows outside the box or missing every interval
 // are culled; the survivors are still tested sample by sample.
+__device__ __forceinline__ bool window_maybe(const Geo& g, const float o[3], const float d[3], int ka, int kz) {
+  bool maybe = false;
+  const float ta = __fmul_rn((float)ka, g.step), tb = __fmul_rn((float)kz, g.step);
+  float lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float pa = __fadd_rn(o[a], __fmul_rn(ta, d[a])), pb = __fadd_rn(o[a], __fmul_rn(tb, d[a]));
+    const float pad = 1e-5f * (1.0f + fmaxf(fabsf(pa), fabsf(pb)));
+    lo[a] = fminf(pa, pb) - pad;
+    hi[a] = fmaxf(pa, pb) + pad;
+  }
+  const bool in_box = hi[0] >= g.lo[0] && lo[0] <= g.hi[0] && hi[1] >= g.lo[1] && lo[1] <= g.hi[1] &&
+                      hi[2] >= g.lo[2] && lo[2] <= g.hi[2];
+  if (in_box) {
+    const int cx0 = min(max((int)floorf(__fmul_rn(__fsub_rn(fmaxf(lo[0], g.lo[0]), g.lo[0]), g.osx)), 0), g.M - 1);
+    const int cx1 = min(max((int)floorf(__fmul_rn(__fsub_rn(fminf(hi[0], g.hi[0]), g.lo[0]), g.osx)), 0), g.M - 1);
+    const int cy0 = min(max((int)floorf(__fmul_rn(__fsub_rn(fmaxf(lo[1], g.lo[1]), g.lo[1]), g.osy)), 0), g.M - 1);
+    const int cy1 = min(max((int)floorf(__fmul_rn(__fsub_rn(fminf(hi[1], g.hi[1]), g.lo[1]), g.osy)), 0), g.M - 1);
+    const int X0 = cx0 >> g.clog2, X1 = cx1 >> g.clog2, Y0 = cy0 >> g.clog2, Y1 = cy1 >> g.clog2;
+    if (X1 - X0 <= 1 && Y1 - Y0 <= 1) {
+      // the common case: at most 2 x 2 coarse cells, read independently
+      const float2 h00 = __ldg(g.chull + X0 * g.Mc + Y0), h01 = __ldg(g.chull + X0 * g.Mc + Y1);
+      const float2 h10 = __ldg(g.chull + X1 * g.Mc + Y0), h11 = __ldg(g.chull + X1 * g.Mc + Y1);
+      const float zl = fminf(fminf(h00.x, h01.x), fminf(h10.x, h11.x));
+      const float zh = fmaxf(fmaxf(h00.y, h01.y), fmaxf(h10.y, h11.y));
+      maybe = zl <= hi[2] && zh >= lo[2];
+    } else if ((X1 - X0 + 1) * (Y1 - Y0 + 1) > 16) {
+      maybe = true;  // unusually long window in cell units: keep it
+    } else {
+      for (int X = X0; X <= X1 && !maybe; X++)
+        for (int Y = Y0; Y <= Y1 && !maybe; Y++) {
+          const float2 h = __ldg(g.chull + X * g.Mc + Y);
+          maybe = h.x <= hi[2] && h.y >= lo[2];
+        }
+    }
+  }
+  return maybe;
+}
 __device__ __forceinline__ unsigned window_mask(const Geo& g, const float o[3], const float d[3], int kb, int kh,
                                                 int lane) {
   const int ka = kb + 32 * lane;
-  bool maybe = false;
-  if (ka <= kh) {
-    const int kz = min(ka + 31, kh);
-    const float ta = __fmul_rn((float)ka, g.step), tb = __fmul_rn((float)kz, g.step);
-    float lo[3], hi[3];
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      const float pa = __fadd_rn(o[a], __fmul_rn(ta, d[a])), pb = __fadd_rn(o[a], __fmul_rn(tb, d[a]));
-      const float pad = 1e-5f * (1.0f + fmaxf(fabsf(pa), fabsf(pb)));
-      lo[a] = fminf(pa, pb) - pad;
-      hi[a] = fmaxf(pa, pb) + pad;
-    }
-    const bool in_box = hi[0] >= g.lo[0] && lo[0] <= g.hi[0] && hi[1] >= g.lo[1] && lo[1] <= g.hi[1] &&
-                        hi[2] >= g.lo[2] && lo[2] <= g.hi[2];
-    if (in_box) {
-      const int cx0 = min(max((int)floorf(__fmul_rn(__fsub_rn(fmaxf(lo[0], g.lo[0]), g.lo[0]), g.osx)), 0), g.M - 1);
-      const int cx1 = min(max((int)floorf(__fmul_rn(__fsub_rn(fminf(hi[0], g.hi[0]), g.lo[0]), g.osx)), 0), g.M - 1);
-      const int cy0 = min(max((int)floorf(__fmul_rn(__fsub_rn(fmaxf(lo[1], g.lo[1]), g.lo[1]), g.osy)), 0), g.M - 1);
-      const int cy1 = min(max((int)floorf(__fmul_rn(__fsub_rn(fminf(hi[1], g.hi[1]), g.lo[1]), g.osy)), 0), g.M - 1);
-      const int X0 = cx0 >> g.clog2, X1 = cx1 >> g.clog2, Y0 = cy0 >> g.clog2, Y1 = cy1 >> g.clog2;
-      if (X1 - X0 <= 1 && Y1 - Y0 <= 1) {
-        // the common case: at most 2 x 2 coarse cells, read independently
-        const float2 h00 = __ldg(g.chull + X0 * g.Mc + Y0), h01 = __ldg(g.chull + X0 * g.Mc + Y1);
-        const float2 h10 = __ldg(g.chull + X1 * g.Mc + Y0), h11 = __ldg(g.chull + X1 * g.Mc + Y1);
-        const float zl = fminf(fminf(h00.x, h01.x), fminf(h10.x, h11.x));
-        const float zh = fmaxf(fmaxf(h00.y, h01.y), fmaxf(h10.y, h11.y));
-        maybe = zl <= hi[2] && zh >= lo[2];
-      } else if ((X1 - X0 + 1) * (Y1 - Y0 + 1) > 16) {
-        maybe = true;  // unusually long window in cell units: keep it
-      } else {
-        for (int X = X0; X <= X1 && !maybe; X++)
-          for (int Y = Y0; Y <= Y1 && !maybe; Y++) {
-            const float2 h = __ldg(g.chull + X * g.Mc + Y);
-            maybe = h.x <= hi[2] && h.y >= lo[2];
-          }
-      }
-    }
-  }
-  return __ballot_sync(kFull, maybe);
+  return __ballot_sync(kFull, ka <= kh && window_maybe(g, o, d, ka, min(ka + 31, kh)));
 }
 
 // Eq. 6 with q = 2; overlapping ramps take the smaller value.  branch: 0 flat,
@@ -466,6 +488,155 @@ __device__ __forceinline__ void gather_features(const Geo& g, const float p[3], 
   grid_stencil<SPARSE>(g, p, goff, gw);
   plane_stencil(g, p, poff, pw);
   gather_texels<FT>(g, goff, gw, poff, pw, t);
+}
+
+// ---------------------------------------------------------------------------
+// The same stencils in even / odd order: along x and y (the slow axes of the
+// arrays) slot 0 is the even index of the cell's two, slot 1 the odd one,
+// whichever is lower.  Four neighbouring samples whose cells differ by one
+// along an axis then read one row in one of the two loads instead of two
+// rows in both (a 256-bit load takes one L1 wavefront per distinct 128-byte
+// line in each group of four lanes).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void even_odd(int i, float f, int idx[2], float w[2], int& odd) {
+  odd = i & 1;
+  idx[0] = (i + 1) & ~1;
+  idx[1] = i | 1;
+  w[0] = odd ? f : 1.0f - f;
+  w[1] = odd ? 1.0f - f : f;
+}
+
+template <bool SPARSE>
+__device__ __forceinline__ void grid_stencil_eo(const Geo& g, const float p[3], int off[8], float w[8], int odd[2]) {
+  int i[3], ix[2], iy[2];
+  float f[3], wx[2], wy[2];
+#pragma unroll
+  for (int a = 0; a < 3; a++) axis_coord(p[a], g.lo[a], g.gs[a], g.L[a], i[a], f[a]);
+  even_odd(i[0], f[0], ix, wx, odd[0]);
+  even_odd(i[1], f[1], iy, wy, odd[1]);
+#pragma unroll
+  for (int c = 0; c < 8; c++) w[c] = wx[(c >> 2) & 1] * wy[(c >> 1) & 1] * ((c & 1) ? f[2] : 1.0f - f[2]);
+  if (!SPARSE) {
+    const int sz = kNch, sy = g.L[2] * kNch, sx = g.L[1] * g.L[2] * kNch;
+#pragma unroll
+    for (int c = 0; c < 8; c++) off[c] = ix[(c >> 2) & 1] * sx + iy[(c >> 1) & 1] * sy + (i[2] + (c & 1)) * sz;
+  } else {
+    // a cell that leaves its brick along x or y has an odd lower index there,
+    // so its corner in the neighbour brick is the even slot
+    const int s = g.blog2, m = (1 << s) - 1;
+    const int lin = ((i[0] >> s) * g.nb[1] + (i[1] >> s)) * g.nb[2] + (i[2] >> s);
+    const int cx = (i[0] & m) == m, cy = (i[1] & m) == m, cz = (i[2] & m) == m;
+    int nb[8];
+    if (cx | cy | cz) {
+      asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=r"(nb[0]), "=r"(nb[1]), "=r"(nb[2]), "=r"(nb[3]), "=r"(nb[4]), "=r"(nb[5]), "=r"(nb[6]),
+                     "=r"(nb[7])
+                   : "l"(g.nbr + 8 * lin));
+    } else {
+      const int o0 = __ldg(g.table + lin) << (3 * s + 3);
+#pragma unroll
+      for (int c = 0; c < 8; c++) nb[c] = o0;
+    }
+    const int lx[2] = {(ix[0] & m) << (2 * s + 3), (ix[1] & m) << (2 * s + 3)};
+    const int ly[2] = {(iy[0] & m) << (s + 3), (iy[1] & m) << (s + 3)};
+    const int lz[2] = {(i[2] & m) << 3, ((i[2] + 1) & m) << 3};
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+      const int dx = (c >> 2) & 1, dy = (c >> 1) & 1, dz = c & 1;
+      const int kx = (dx ^ 1) & cx, ky = (dy ^ 1) & cy, kz = dz & cz;
+      const int z0 = kz ? nb[1] : nb[0], z1 = kz ? nb[3] : nb[2], z2 = kz ? nb[5] : nb[4], z3 = kz ? nb[7] : nb[6];
+      const int y0 = ky ? z1 : z0, y1 = ky ? z3 : z2;
+      const int b = kx ? y1 : y0;
+      off[c] = b + lx[dx] + ly[dy] + lz[dz];  // negative through an unstored brick
+    }
+    check_unallocated(g, off);
+  }
+}
+
+__device__ __forceinline__ void plane_stencil_eo(const Geo& g, const float p[3], int off[12], float w[12], int odd[2]) {
+  int i[3], ix[2], iy[2];
+  float f[3], wx[2], wy[2];
+#pragma unroll
+  for (int a = 0; a < 3; a++) axis_coord(p[a], g.lo[a], g.ps[a], g.R[a], i[a], f[a], a == 2 ? g.pzoff : 0.0f);
+  even_odd(i[0], f[0], ix, wx, odd[0]);
+  even_odd(i[1], f[1], iy, wy, odd[1]);
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const int du = (c >> 1) & 1, dv = c & 1;
+    off[c] = (ix[du] * g.R[1] + i[1] + dv) * kNch;
+    w[c] = wx[du] * (dv ? f[1] : 1.0f - f[1]);
+    off[4 + c] = (ix[du] * g.R[2] + i[2] + dv) * kNch;
+    w[4 + c] = wx[du] * (dv ? f[2] : 1.0f - f[2]);
+    off[8 + c] = (iy[du] * g.R[2] + i[2] + dv) * kNch;
+    w[8 + c] = wy[du] * (dv ? f[2] : 1.0f - f[2]);
+  }
+}
+
+// The weighted sum of Eq. 2 over an even / odd stencil, two channels per
+// packed FP32 FMA.  DENSITY: also the density channel summed in the order of
+// gather_features (lower index first), bit for bit its t[0].
+template <bool SPARSE, bool DENSITY>
+__device__ __forceinline__ void gather_features_eo(const Geo& g, const float p[3], float t[8], float& t0) {
+  int goff[8], poff[12], odd[2][2];
+  float gw[8], pw[12], v0[20];
+  grid_stencil_eo<SPARSE>(g, p, goff, gw, odd[0]);
+  plane_stencil_eo(g, p, poff, pw, odd[1]);
+  float2 t2[4];
+#pragma unroll
+  for (int c = 0; c < 4; c++) t2[c] = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int c = 0; c < 8; c++) {
+    float v[8];
+    if (DENSITY) v0[c] = 0.0f;
+    if (goff[c] >= 0 && check_range(g, 0, goff[c])) {
+      Texel<float>::load(g.grid, goff[c], v);
+      fma8x2(t2, gw[c], v);
+      if (DENSITY) v0[c] = v[0];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const void* P = plane_base(g, q);
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      float v[8];
+      if (DENSITY) v0[8 + 4 * q + c] = 0.0f;
+      if (!check_range(g, 1 + q, poff[4 * q + c])) continue;
+      Texel<float>::load(P, poff[4 * q + c], v);
+      fma8x2(t2, pw[4 * q + c], v);
+      if (DENSITY) v0[8 + 4 * q + c] = v[0];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    t[2 * c] = t2[c].x;
+    t[2 * c + 1] = t2[c].y;
+  }
+  if (DENSITY) {
+    // (an unstored corner adds w * 0 here and nothing there: the same sum)
+    t0 = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+      float w[2], v[2];
+#pragma unroll
+      for (int b = 0; b < 2; b++) {  // b: the slot along x
+        const int lo = 4 * b + (c & 3), hi = lo ^ 2;
+        w[b] = odd[0][1] ? gw[hi] : gw[lo];
+        v[b] = odd[0][1] ? v0[hi] : v0[lo];
+      }
+      const int x = c >> 2;
+      t0 = fmaf(odd[0][0] ? w[x ^ 1] : w[x], odd[0][0] ? v[x ^ 1] : v[x], t0);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const bool o = odd[1][q == 2 ? 1 : 0];
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const int a = 4 * q + c, b = a ^ 2;
+        t0 = fmaf(o ? pw[b] : pw[a], o ? v0[8 + b] : v0[8 + a], t0);
+      }
+    }
+  }
 }
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }

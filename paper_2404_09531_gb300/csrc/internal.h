@@ -73,8 +73,13 @@ cudaError_t launch_march_bwd(const omerf_scene* s, const float* rays, const floa
                              float* g_grid, float* g_xy, float* g_xz, float* g_yz, float* g_occ,
                              float* g_mlp, float* loss, cudaStream_t stream);
 
-cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int n_cams, long n_super, long n,
+cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int n_cams, int lanes, long n_super, long n,
                                   float* rgb, int* count, cudaStream_t stream);
+
+// Lanes that march one ray of a camera render of n rays (0: the packed
+// queue of march_fwd.cu), and the pixels of the super-tile a CTA takes.
+int cam_lanes(const omerf_scene* s, long n);
+void cam_super(int lanes, int& w, int& h);
 
 int persistent_blocks(const void* kernel, int threads, size_t smem, int num_sms);
 

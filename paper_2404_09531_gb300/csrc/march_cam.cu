@@ -1,0 +1,466 @@
+// march_cam.cu -- FP32 camera render, a fixed set of lanes per ray (sm_103a).
+//
+// The L1 data pipe bounds the render: a 256-bit texel load takes one
+// wavefront per distinct 128-byte line in each group of four lanes, 20 loads
+// per sample, and the packed queue of march_fwd.cu adds a quarter more for
+// its shared-memory queue and segmented scans.  Neighbouring pixels march
+// through neighbouring texels and evaluate nearly the same number of samples
+// (95 % of the lanes stay busy when the 32 rays of an 8 x 4 tile are marched
+// one per lane), so a camera needs no queue: every ray is marched by its own
+// G lanes, which keep its transmittance and sums in registers.
+//   G = 1  one lane per ray; the four lanes of a 2 x 2 pixel quad share a
+//          lattice frame, so the lanes of a load group sample one depth (254
+//          wavefronts per 32 samples by a replay, 293 without the frame)
+//   G = 4, 8  the lanes of a ray take consecutive lattice indices: a ray's
+//          serial chain is 4 or 8 times shorter and there are 4 or 8 times
+//          the warps, for images too small to fill the chip with G = 1
+// A frame skips the 32-index windows that the coarse occupancy grid rules
+// out.  Texel pairs are read in even / odd order (216 wavefronts, see
+// even_odd) with two channels per FMA.  All forms composite a ray's samples
+// one after the other in the same order, so a pixel does not depend on G, nor
+// on whether counts are wanted.
+//
+// Measured on a GB300, 512 x 512 x 32 city, against the packed queue:
+// 8 x 1920x1080 29.4 -> 21.0 ms (L1 pipe 86 % busy), 1920x1080 3.80 -> 2.73
+// ms (G = 4: 3.11), 641x361 0.84 -> 0.45 ms (G = 8: 0.50, G = 1: 0.91),
+// 64x64 of the 64 x 64 x 16 field 0.155 -> 0.058 ms (G = 4: 0.080).
+//
+// Sample counts are those of the packed queue, which training and ray lists
+// use, also where rounding decides them.  The two forms multiply a ray's
+// transmittance in different orders: where counts are wanted the density is
+// also summed in the queue's order, its transmittance decides the count, and
+// a ray that passes the termination threshold within the products' rounding
+// (about 1 of 10^5) is counted again by marching its tile with the queue.
+#include "march_fwd.cuh"
+
+namespace omerf {
+
+// Warps per CTA and the pixels of its super-tile (whole or half 8 x 4 tiles).
+// CTAs of 4 warps wait less for their slowest tile than CTAs of 8 (2.96
+// against 3.10 ms per 1080p frame; 2 warps 3.05).
+template <int G>
+struct CamShape;
+template <>
+struct CamShape<1> {
+  static constexpr int kWarps = 4, kW = 16, kH = 8;
+};
+template <>
+struct CamShape<4> {
+  static constexpr int kWarps = 4, kW = 8, kH = 4;
+};
+template <>
+struct CamShape<8> {
+  static constexpr int kWarps = 4, kW = 4, kH = 4;
+};
+
+// Pixel of a lane's ray inside the super-tile.
+template <int G>
+__device__ __forceinline__ void lane_pixel(int warp, int lane, int& x, int& y) {
+  if (G == 1) {  // 8 x 4 pixels per warp, quads of 2 x 2
+    const int q = lane >> 2, j = lane & 3;
+    x = (warp & 1) * 8 + (q & 3) * 2 + (j & 1);
+    y = (warp >> 1) * 4 + (q >> 2) * 2 + (j >> 1);
+  } else if (G == 4) {  // 4 x 2 pixels per warp
+    const int r = lane >> 2;
+    x = (warp & 1) * 4 + (r & 3);
+    y = (warp >> 1) * 2 + (r >> 2);
+  } else {  // 2 x 2 pixels per warp
+    const int r = lane >> 3;
+    x = (warp & 1) * 2 + (r & 1);
+    y = (warp >> 1) * 2 + (r >> 1);
+  }
+}
+
+// mlp_forward_padded with the units of each layer spread over the G lanes of
+// a ray (every unit summed in the same order): output j is lane j's return
+// value, j < 3.  All lanes of the warp call it.
+template <int G>
+__device__ __forceinline__ float mlp_group(const float* __restrict__ W, const float F[7], const float d[3], int j) {
+  float sc[(12 + G - 1) / G][2];
+#pragma unroll
+  for (int i = 0; i < (12 + G - 1) / G; i++) {
+    const int m = min(i * G + j, 11), k = m / 3, a = m - 3 * k;
+    const float da = a == 0 ? d[0] : (a == 1 ? d[1] : d[2]);
+    sincosf((float)(1 << k) * da, &sc[i][0], &sc[i][1]);
+  }
+  float x[36];
+#pragma unroll
+  for (int i = 0; i < 7; i++) x[i] = F[i];
+#pragma unroll
+  for (int a = 0; a < 3; a++) x[7 + a] = d[a];
+#pragma unroll
+  for (int m = 0; m < 12; m++) {
+    const int k = m / 3, a = m % 3;
+    x[10 + 6 * k + a] = __shfl_sync(kFull, sc[m / G][0], m % G, G);
+    x[10 + 6 * k + 3 + a] = __shfl_sync(kFull, sc[m / G][1], m % G, G);
+  }
+  x[34] = 0.0f;
+  x[35] = 0.0f;
+  float h[16 / G];
+#pragma unroll
+  for (int i = 0; i < 16 / G; i++) {
+    const int u = i * G + j;
+    const float4* w = reinterpret_cast<const float4*>(W + kSW1 + 36 * u);
+    float a = W[kSB1 + u];
+#pragma unroll
+    for (int q = 0; q < 9; q++) a = dot4(w[q], x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3], a);
+    h[i] = fmaxf(a, 0.0f);
+  }
+  float h1[16];
+#pragma unroll
+  for (int u = 0; u < 16; u++) h1[u] = __shfl_sync(kFull, h[u / G], u % G, G);
+#pragma unroll
+  for (int i = 0; i < 16 / G; i++) {
+    const int u = i * G + j;
+    const float4* w = reinterpret_cast<const float4*>(W + kSW2 + 16 * u);
+    float a = W[kSB2 + u];
+#pragma unroll
+    for (int q = 0; q < 4; q++) a = dot4(w[q], h1[4 * q], h1[4 * q + 1], h1[4 * q + 2], h1[4 * q + 3], a);
+    h[i] = fmaxf(a, 0.0f);
+  }
+  float h2[16];
+#pragma unroll
+  for (int u = 0; u < 16; u++) h2[u] = __shfl_sync(kFull, h[u / G], u % G, G);
+  const int o = min(j, 2);
+  const float4* w = reinterpret_cast<const float4*>(W + kSW3 + 16 * o);
+  float a = W[kSB3 + o];
+#pragma unroll
+  for (int q = 0; q < 4; q++) a = dot4(w[q], h2[4 * q], h2[4 * q + 1], h2[4 * q + 2], h2[4 * q + 3], a);
+  return sigmoidf_(a);
+}
+
+// The bits of a ballot that belong to the lanes of this lane's ray.
+template <int G>
+__device__ __forceinline__ unsigned hits_of(bool v, int base) {
+  return (__ballot_sync(kFull, v) >> base) & ((1u << G) - 1u);
+}
+
+// A ray's transmittance T carried through its G lanes' opacities in lane
+// order: returns the transmittance before this lane's sample; `last` is the
+// lane whose sample takes it below thr, G if none does.
+template <int G>
+__device__ __forceinline__ float chain(float T, float ah, bool hit, int j, int base, float thr, int& last) {
+  const float om = __fsub_rn(1.0f, ah);
+#pragma unroll
+  for (int i = 0; i < G - 1; i++) {
+    const float v = __shfl_sync(kFull, om, i, G);
+    if (i < j) T = __fmul_rn(T, v);
+  }
+  const unsigned below = hits_of<G>(hit && __fmul_rn(T, om) < thr, base);
+  last = below ? __ffs(below) - 1 : G;
+  return T;
+}
+
+// The camera of super-tile sb, its pixel origin and first ray.
+template <int G>
+__device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb, int& x0, int& y0, long& ray0) {
+  const Cam* cam = &a.cam;
+  int super_x = a.super_x;
+  ray0 = 0;
+  if (a.n_cams > 0) {
+    int c = 0;
+    while (c + 1 < a.n_cams && (long long)sb >= a.cams[c + 1].super_start) c++;
+    const CamRec& cr = a.cams[c];
+    sb = (unsigned)((long long)sb - cr.super_start);
+    cam = &cr.cam;
+    super_x = cr.super_x;
+    ray0 = (long)cr.ray_start;
+  }
+  x0 = (int)(sb % (unsigned)super_x) * CamShape<G>::kW;
+  y0 = (int)(sb / (unsigned)super_x) * CamShape<G>::kH;
+  return *cam;
+}
+
+// March one 8 x 4 tile with the packed queue (32 rays of one warp) and write
+// the sample counts of the pixels whose bit is set in `want` (bit 8 y + x).
+template <class FT, bool SPARSE, int G>
+__device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, WarpMarch<false>& ws, unsigned sb, int tx,
+                                            int ty, unsigned want) {
+  const int lane = threadIdx.x & 31;
+  int x0, y0;
+  long ray0;
+  const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
+  const int px = ((x0 >> 3) + tx) * 8 + (lane & 7), py = ((y0 >> 2) + ty) * 4 + (lane >> 3);
+  const bool valid = px < cam.width && py < cam.height;
+  float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
+  if (valid) camera_ray(cam, px, py, o, d);
+  int klo = 0, khi = -1;
+  const bool any = valid && lattice_range(g, o, d, klo, khi);
+  march_bundle<FT, SPARSE>(g, lane, o, d, klo, khi, any, ws);
+  if (valid && ((want >> lane) & 1u)) a.count[ray0 + (long)py * cam.width + px] = ws.s.cnt[lane];
+}
+
+// 7 CTAs of 4 warps (72 registers) per SM: 2.91 ms per 1080p frame, 2.90 with
+// 6, 3.07 with 8, 2.94 with 5.
+template <class FT, bool SPARSE, int G, bool COUNT>
+__global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
+    march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
+  constexpr int kWarps = CamShape<G>::kWarps;
+  constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
+  constexpr unsigned kFrameMask = (1u << kFrame) - 1u;
+  constexpr int kTilesX = (CamShape<G>::kW + 7) / 8, kTilesY = (CamShape<G>::kH + 3) / 4;
+  __shared__ __align__(16) float sW[kSmemMlp];
+  __shared__ typename std::conditional<COUNT, WarpMarch<false>, int>::type sMarch;
+  __shared__ unsigned sWork[2], sAmb[kTilesX * kTilesY];
+  load_mlp_padded(g.mlp, sW);
+  if (COUNT && threadIdx.x < kTilesX * kTilesY) sAmb[threadIdx.x] = 0u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int base = lane & ~(kFrame - 1), j = G == 1 ? 0 : lane & (G - 1);
+  if (threadIdx.x == 0) sWork[0] = atomicAdd(a.counter, 1u);
+  __syncthreads();
+  for (int it = 0;; it ^= 1) {
+    const unsigned sb = sWork[it];
+    if (sb >= a.n_super) break;
+    if (threadIdx.x == 0) sWork[it ^ 1] = atomicAdd(a.counter, 1u);
+
+    int sx, sy, x0, y0;
+    long ray0;
+    lane_pixel<G>(warp, lane, sx, sy);
+    float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
+    const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
+    const int px = x0 + sx, py = y0 + sy;
+    const bool valid = px < cam.width && py < cam.height;
+    const long rid = ray0 + (long)py * cam.width + px;
+    if (valid) camera_ray(cam, px, py, o, d);
+    int klo = 0, khi = -1;
+    bool alive = valid && lattice_range(g, o, d, klo, khi);
+    if (!alive) {
+      klo = 0x7fffffff;
+      khi = -1;
+    }
+    // the common lattice frame
+    int k = klo, ke = khi;
+    if (G == 1) {
+      k = min(k, __shfl_xor_sync(kFull, k, 1));
+      k = min(k, __shfl_xor_sync(kFull, k, 2));
+      ke = max(ke, __shfl_xor_sync(kFull, ke, 1));
+      ke = max(ke, __shfl_xor_sync(kFull, ke, 2));
+    }
+    int wb = k;
+    unsigned wm = 0;
+    bool need_mask = true, amb = false, done = false, counted = false;
+    float T = 1.0f, Tc = 1.0f, F[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    int seen = 0, cnt = 0, ccell = -1;
+    float2 zb = make_float2(0.0f, 0.0f);
+    while (__any_sync(kFull, k <= ke)) {
+      // advance every frame to its next lattice index (or G of them) at which
+      // a ray is evaluated
+      bool hit = false, need = k <= ke;
+      unsigned hits = 0;
+      float p[3] = {0.0f, 0.0f, 0.0f};
+      while (__any_sync(kFull, need)) {
+        if (__any_sync(kFull, need_mask)) {
+          // windows of 32 indices that the coarse grid cannot rule out
+          unsigned m = 0;
+          if (need_mask && alive) {
+            const int nw = min((ke - wb) >> 5, 31);
+            for (int jw = j; jw <= nw; jw += G) {
+              const int ka = max(wb + 32 * jw, klo), kz = min(wb + 32 * jw + 31, khi);
+              if (ka <= kz && window_maybe(g, o, d, ka, kz)) m |= 1u << jw;
+            }
+          }
+#pragma unroll
+          for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
+          if (need_mask) wm = m;
+          need_mask = false;
+        }
+        bool h = false;
+        if (need) {
+          const int off = k - wb;
+          if (off >= 1024) {
+            wb = k;
+            need_mask = true;
+          } else {
+            const unsigned rem = wm & (~0u << (off >> 5));
+            const int jn = __ffs(rem) - 1;
+            if (rem == 0) {
+              k = wb + 1024;
+            } else {
+              if (jn > (off >> 5)) k = wb + 32 * jn;
+              const int kk = k + j;
+              h = alive && kk >= klo && kk <= khi && lattice_test_cached(g, o, d, kk, p, zb, ccell);
+              k += G;
+            }
+          }
+        }
+        const unsigned hb = __ballot_sync(kFull, h);
+        if (need) {
+          hit = h;
+          hits = (hb >> base) & kFrameMask;
+          need = hits == 0u && k <= ke;
+        }
+      }
+      if (G == 1) {
+        if (hit) {
+          float t[8], t0;
+          gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
+          SampleAct s;
+          activate(g, t, p[2], zb, s);
+          seen++;
+          if (!COUNT || !done) {
+            const float w = __fmul_rn(T, s.ah);
+#pragma unroll
+            for (int c = 0; c < 7; c++) F[c] = fmaf(w, s.x[c], F[c]);
+            T = __fmul_rn(T, __fsub_rn(1.0f, s.ah));
+            done = T < g.t_thr;
+          }
+          if (COUNT && !counted) {
+            t[0] = t0;
+            activate(g, t, p[2], zb, s);
+            Tc = __fmul_rn(Tc, __fsub_rn(1.0f, s.ah));
+            cnt = seen;
+            counted = Tc < g.t_thr;
+            amb |= fabsf(Tc - g.t_thr) < g.t_thr * ambiguity(cnt);
+          }
+          alive = seen < g.n_max && !(done && (!COUNT || counted));
+        }
+        const unsigned am = __ballot_sync(kFull, alive);
+        if (((am >> base) & kFrameMask) == 0u) k = ke + 1;
+      } else {
+        const int rank = __popc(hits & ((1u << j) - 1u));  // this frame's samples before this lane's
+        hit = hit && seen + rank < g.n_max;
+        SampleAct s;
+        s.ah = 0.0f;
+        float ahc = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 7; c++) s.x[c] = 0.0f;
+        if (hit) {
+          float t[8], t0;
+          gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
+          activate(g, t, p[2], zb, s);
+          if (COUNT) {
+            SampleAct sc;
+            t[0] = t0;
+            activate(g, t, p[2], zb, sc);
+            ahc = sc.ah;
+          }
+        }
+        if (!COUNT || __any_sync(kFull, !done)) {
+          // transmittance before each lane's sample, in lattice order
+          int last;
+          const float Ta = chain<G>(T, s.ah, hit, j, base, g.t_thr, last);
+          const unsigned kept = hits_of<G>(hit && !done && j <= last, base);
+          const float w = __fmul_rn(Ta, s.ah);
+#pragma unroll
+          for (int i = 0; i < G; i++) {
+            const float wi = __shfl_sync(kFull, w, i, G);
+#pragma unroll
+            for (int c = 0; c < 7; c++) {
+              const float xi = __shfl_sync(kFull, s.x[c], i, G);
+              if ((kept >> i) & 1u) F[c] = fmaf(wi, xi, F[c]);
+            }
+          }
+          const float Tn = __shfl_sync(kFull, __fmul_rn(Ta, __fsub_rn(1.0f, s.ah)), min(last, G - 1), G);
+          if (!done) T = Tn;
+          done = done || last < G;
+        }
+        if (COUNT && __any_sync(kFull, !counted)) {
+          int last;
+          const float Ta = __fmul_rn(chain<G>(Tc, ahc, hit, j, base, g.t_thr, last), __fsub_rn(1.0f, ahc));
+          const bool kept = hit && !counted && j <= last;
+          const int n = __popc(hits_of<G>(kept, base));
+          if (!counted) cnt = seen + n;
+          amb |= kept && fabsf(Ta - g.t_thr) < g.t_thr * ambiguity(cnt);
+          const float Tn = __shfl_sync(kFull, Ta, min(last, G - 1), G);
+          if (!counted) Tc = Tn;
+          counted = counted || last < G;
+        }
+        seen += __popc(hits_of<G>(hit, base));
+        if (seen >= g.n_max || (done && (!COUNT || counted))) {
+          alive = false;
+          k = ke + 1;
+        }
+      }
+    }
+
+    float out[3];
+    if (G == 1) {
+      if (valid) {
+        float yd[3] = {0.0f, 0.0f, 0.0f};
+        if (seen > 0) mlp_forward_padded(sW, F, d, yd);
+#pragma unroll
+        for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T, g.bg[c], F[c] + yd[c]) : g.bg[c];
+#pragma unroll
+        for (int c = 0; c < 3; c++) a.rgb[3 * rid + c] = out[c];
+        if (COUNT) a.count[rid] = cnt;
+      }
+    } else {
+      float y = 0.0f;
+      if (__any_sync(kFull, seen > 0)) y = mlp_group<G>(sW, F, d, j);
+      if (valid && j < 3) {
+        const float Fj = j == 0 ? F[0] : (j == 1 ? F[1] : F[2]);
+        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T, g.bg[j], Fj + y) : g.bg[j];
+        if (COUNT && j == 0) a.count[rid] = cnt;
+      }
+    }
+    if constexpr (COUNT) {
+      if (amb && valid) {
+        const int tx = (x0 + sx) / 8 - x0 / 8, ty = (y0 + sy) / 4 - y0 / 4;
+        atomicOr(&sAmb[ty * kTilesX + tx], 1u << (((py & 3) << 3) | (px & 7)));
+      }
+      __syncthreads();
+      if (warp == 0) {
+        // rays whose transmittance passed the termination threshold within
+        // rounding: count their tile's samples again
+#pragma unroll 1
+        for (int t = 0; t < kTilesX * kTilesY; t++) {
+          const unsigned want = sAmb[t];
+          if (want) {
+            resolve_counts<FT, SPARSE, G>(g, a, sMarch, sb, t % kTilesX, t / kTilesX, want);
+            __syncwarp();
+            if (lane == 0) sAmb[t] = 0u;
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <class FT, bool SPARSE, int G, bool COUNT>
+static cudaError_t launch_cam_variant(const omerf_scene* s, const FwdArgs& a, cudaStream_t stream) {
+  auto kern = march_cam_kernel<FT, SPARSE, G, COUNT>;
+  constexpr int threads = 32 * CamShape<G>::kWarps;
+  static std::atomic<int> blocks[64];  // per device: resident CTAs of this variant
+  const int dev = s->device & 63;
+  int nb = blocks[dev].load(std::memory_order_relaxed);
+  if (nb == 0) {
+    nb = persistent_blocks((const void*)kern, threads, 0, s->num_sms);
+    blocks[dev].store(nb, std::memory_order_relaxed);
+  }
+  const int grid = (int)(a.n_super < nb ? a.n_super : nb);
+  kern<<<grid < 1 ? 1 : grid, threads, 0, stream>>>(s->geo, a);
+  return cudaGetLastError();
+}
+
+template <int G, bool COUNT>
+static cudaError_t launch_cam_group(const omerf_scene* s, const FwdArgs& a, cudaStream_t stream) {
+  return s->desc.brick > 0 ? launch_cam_variant<float, true, G, COUNT>(s, a, stream)
+                           : launch_cam_variant<float, false, G, COUNT>(s, a, stream);
+}
+
+// The lines lie where the measured times cross (us with 8 / 4 / 1 lanes; city
+// unless said): 57,600 rays 212 / 286 / 781, 129,600 rays 343 / 350 / 865,
+// 230,400 rays 542 / 478 / 998, 921,600 rays 1935 / 1520 / 1593, 1,048,576
+// rays (field) 996 / 721 / 604, 1,398,784 rays 3183 / 2450 / 2212.  A BF16
+// scene keeps the packed queue: its deferred MLP rounds F to bfloat16, so sums
+// in another order would move pixels by a step of that rounding.
+int cam_lanes(const omerf_scene* s, long n) {
+  if (s->desc.feat_dtype != OMERF_F32) return 0;
+  return n < (1 << 17) ? 8 : (n < (1 << 20) ? 4 : 1);
+}
+
+void cam_super(int lanes, int& w, int& h) {
+  w = lanes == 0 ? 16 : (lanes == 1 ? CamShape<1>::kW : (lanes == 4 ? CamShape<4>::kW : CamShape<8>::kW));
+  h = lanes == 0 ? 16 : (lanes == 1 ? CamShape<1>::kH : (lanes == 4 ? CamShape<4>::kH : CamShape<8>::kH));
+}
+
+cudaError_t launch_render_cam(const omerf_scene* s, const FwdArgs& a, int lanes, cudaStream_t stream) {
+  if (a.count)
+    return lanes == 1 ? launch_cam_group<1, true>(s, a, stream)
+                      : (lanes == 4 ? launch_cam_group<4, true>(s, a, stream) : launch_cam_group<8, true>(s, a, stream));
+  return lanes == 1 ? launch_cam_group<1, false>(s, a, stream)
+                    : (lanes == 4 ? launch_cam_group<4, false>(s, a, stream) : launch_cam_group<8, false>(s, a, stream));
+}
+
+}  // namespace omerf

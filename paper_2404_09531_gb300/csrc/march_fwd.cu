@@ -20,131 +20,9 @@
 
 #include <type_traits>
 
-#include "internal.h"
-#include "mlp_mma.cuh"
-#include "packed.cuh"
+#include "march_fwd.cuh"
 
 namespace omerf {
-
-// Per-warp shared state of the packed march of one bundle of 32 rays.
-struct MarchState {
-  WarpQueue q;
-  float F[32][8];    // per-ray accumulated [sum w c^d, sum w f]
-  float T[32];       // per-ray transmittance so far
-  int cnt[32];       // per-ray evaluated samples
-};
-// With the tensor-core MLP the whole march state doubles as the MLP staging
-// area: the epilogue copies each ray's F, T and count to registers before it
-// stages the MLP rows, and the next bundle starts after a CTA barrier.  The
-// smaller per-warp footprint lets the BF16 render take a smaller
-// shared-memory carveout, leaving more of the SM's SRAM to L1.
-template <bool MMA>
-struct WarpMarch {
-  MarchState s;
-};
-template <>
-struct WarpMarch<true> {
-  union {
-    MarchState s;
-    MlpStage m;
-  };
-};
-
-// March the 32 rays of a bundle (lane r owns ray r: o, d, [klo, khi]).
-//
-// fill:    evaluated samples of consecutive rays are queued, 32 at a time
-//          (packed.cuh);
-// process: the 32 queued samples are gathered and activated in parallel;
-//          compositing is a segmented lane scan (segments = rays) of
-//          1 - alpha_hat, early termination is resolved per segment, and
-//          the weighted features are summed per segment into the ray's
-//          accumulator.
-// On return ws.s.F / ws.s.T / ws.s.cnt hold every ray's F, T_N and sample count.
-template <class FT, bool SPARSE, class WS>
-__device__ __forceinline__ void march_bundle(const Geo& g, int lane, const float o[3], const float d[3], int klo,
-                                             int khi, bool any, WS& ws) {
-#pragma unroll
-  for (int c = 0; c < 8; c++) ws.s.F[lane][c] = 0.0f;
-  ws.s.T[lane] = 1.0f;
-  ws.s.cnt[lane] = 0;
-  ws.s.q.ro[lane] = make_float4(o[0], o[1], o[2], __int_as_float(klo));
-  ws.s.q.rd[lane] = make_float4(d[0], d[1], d[2], __int_as_float(khi));
-  ws.s.q.cap[lane] = g.n_max;
-  unsigned pend = __ballot_sync(kFull, any);
-  FillState f;
-  __syncwarp();
-  while (pend) {
-    const int nq = fill_queue(g, lane, pend, f, ws.s.q);
-    if (nq == 0) break;
-    const bool act = lane < nq;
-    const float4 qa = ws.s.q.a[lane], qb = ws.s.q.b[lane];
-    const int r = act ? __float_as_int(qb.y) : 32;
-    SampleAct s;
-    s.ah = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 7; c++) s.x[c] = 0.0f;
-    if (act) {
-      const float p[3] = {qa.x, qa.y, qa.z};
-      float t[8];
-      gather_features<FT, SPARSE>(g, p, t);
-      activate(g, t, p[2], make_float2(qa.w, qb.x), s);
-    }
-    bool head;
-    const int segstart = segment_start(lane, r, head);
-    // transmittance: segmented inclusive product scan of (1 - alpha_hat)
-    const float P = seg_prod_scan(1.0f - s.ah, lane, segstart);
-    float Pex = __shfl_up_sync(kFull, P, 1);
-    if (head) Pex = 1.0f;
-    const float Tprev = act ? ws.s.T[r] : 1.0f;
-    const float Ti = Tprev * Pex, Tn = Tprev * P;
-    // early termination: the first sample of a segment whose T drops below t_thr ends the ray
-    const bool term = act && Tn < g.t_thr;
-    const unsigned tm = __ballot_sync(kFull, term);
-    const unsigned seglt = lanemask_lt() & ~((1u << segstart) - 1u);
-    const bool dropped = (tm & seglt) != 0u;
-    const bool ok = act && !dropped;
-    const float w = ok ? Ti * s.ah : 0.0f;
-    float wx[7];
-#pragma unroll
-    for (int c = 0; c < 7; c++) wx[c] = w * s.x[c];
-    seg_sum_scan7(wx, lane, segstart);
-    const unsigned okm = __ballot_sync(kFull, ok);
-    const int rnext = __shfl_down_sync(kFull, r, 1);
-    const bool tail = act && (lane == 31 || rnext != r);
-    const unsigned segle = lanemask_le() & ~((1u << segstart) - 1u);
-    if (tail) {
-#pragma unroll
-      for (int c = 0; c < 7; c++) ws.s.F[r][c] += wx[c];
-      ws.s.cnt[r] += __popc(okm & segle);
-      if (!(tm & segle)) ws.s.T[r] = Tn;
-    }
-    const bool first_term = term && !dropped;
-    if (first_term) ws.s.T[r] = Tn;
-    pend &= ~__reduce_or_sync(kFull, first_term ? (1u << r) : 0u);
-    __syncwarp();
-  }
-}
-
-struct FwdArgs {
-  Cam cam;
-  int use_cam, super_x;
-  const float* rays;
-  long n, n_super;
-  float* rgb;
-  int* count;
-  // training
-  const float* target;
-  const float* dirs;
-  int K;
-  float lam_rgb, lam_smooth;  // already divided by n
-  float* saved;
-  float* loss;
-  unsigned* counter;
-  // multi-camera render (n_cams > 0): device camera records, super-tiles in
-  // camera order
-  const CamRec* cams;
-  int n_cams;
-};
 
 #ifndef OMERF_FWD_MINB
 #define OMERF_FWD_MINB 3  // resident CTAs per SM the register budget is sized for
@@ -360,11 +238,15 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
                              float* saved, float* loss, cudaStream_t stream) {
   FwdArgs a{};
   const bool train = saved != nullptr;
+  int lanes = 0;
   if (cam) {
     a.cam = *cam;
     a.use_cam = 1;
-    a.super_x = (cam->width + 15) / 16;
-    a.n_super = (long)a.super_x * ((cam->height + 15) / 16);
+    int sw, sh;
+    lanes = cam_lanes(s, n);
+    cam_super(lanes, sw, sh);
+    a.super_x = (cam->width + sw - 1) / sw;
+    a.n_super = (long)a.super_x * ((cam->height + sh - 1) / sh);
   } else {
     a.use_cam = 0;
     a.n_super = (n + 255) / 256;
@@ -384,6 +266,7 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
   a.loss = loss;
   if (a.n_super == 0) return cudaSuccess;
   a.counter = next_counter(s, stream);
+  if (lanes > 0) return launch_render_cam(s, a, lanes, stream);
   const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
   const bool sparse = s->desc.brick > 0;
   if (train && loss) {
@@ -403,7 +286,7 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
 }
 
 
-cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int n_cams, long n_super, long n,
+cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int n_cams, int lanes, long n_super, long n,
                                   float* rgb, int* count, cudaStream_t stream) {
   FwdArgs a{};
   a.use_cam = 1;
@@ -415,6 +298,7 @@ cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int 
   a.count = count;
   if (a.n_super == 0) return cudaSuccess;
   a.counter = next_counter(s, stream);
+  if (lanes > 0) return launch_render_cam(s, a, lanes, stream);
   const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
   const bool sparse = s->desc.brick > 0;
   if (bf16) return sparse ? launch_variant<__nv_bfloat16, true, false>(s, a, stream)

@@ -743,21 +743,26 @@ omerf_status omerf_render_cameras(const omerf_scene* s, const omerf_camera* cams
     const int m = std::min(kMaxCams, n_cams - c0);
     CamRec rec[kMaxCams];
     long supers = 0, rays = 0;
+    for (int c = 0; c < m; c++) rays += (long)cams[c0 + c].width * cams[c0 + c].height;
+    const int lanes = cam_lanes(s, rays);
+    int sw, sh;
+    cam_super(lanes, sw, sh);
+    rays = 0;
     for (int c = 0; c < m; c++) {
       const omerf_camera& k = cams[c0 + c];
       rec[c].cam = to_cam(&k);
-      rec[c].super_x = (k.width + 15) / 16;
+      rec[c].super_x = (k.width + sw - 1) / sw;
       rec[c].super_start = supers;
       rec[c].ray_start = rays;
       rec[c].pad = 0;
-      supers += (long)rec[c].super_x * ((k.height + 15) / 16);
+      supers += (long)rec[c].super_x * ((k.height + sh - 1) / sh);
       rays += (long)k.width * k.height;
     }
     OMERF_LAUNCH_FAULT();
     // pageable source: the copy is staged before the call returns
     cudaError_t e = cudaMemcpyAsync(s->cams, rec, m * sizeof(CamRec), cudaMemcpyHostToDevice, cs);
     if (e != cudaSuccess) return cuda_fail(e, "camera upload");
-    e = launch_march_fwd_cams(s, s->cams, m, supers, rays, static_cast<float*>(rd) + 3 * ray0,
+    e = launch_march_fwd_cams(s, s->cams, m, lanes, supers, rays, static_cast<float*>(rd) + 3 * ray0,
                               cd ? static_cast<int32_t*>(cd) + ray0 : nullptr, cs);
     if (e != cudaSuccess) return cuda_fail(e, "render launch");
     ray0 += rays;
