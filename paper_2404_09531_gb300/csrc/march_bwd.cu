@@ -27,9 +27,6 @@
 namespace omerf {
 
 constexpr int kBwdThreads = 128;   // 4 warps per CTA
-#ifndef OMERF_FOLD
-#define OMERF_FOLD 3       // lanes folded into one reduction
-#endif
 constexpr int kRow = 101;          // staged floats per ray: x 34, h1 16, h2 16, g1 16, g2 16, g3 3
 
 struct BwdArgs {
@@ -422,24 +419,90 @@ __device__ __forceinline__ void warp_mlp_input_grad(float* __restrict__ rows, co
   for (int i = 0; i < 7; i++) gF[i] += row[i];
 }
 
-// Pair folding by stencil: lanes whose samples share the key (the base grid
-// vertex, or a plane's base texel) share every texel of that stencil, so a
-// lane at an even position of a run of equal keys adds its right neighbour's
-// contribution and the neighbour issues nothing.
-__device__ __forceinline__ void pair_fold_info(int key, int lane, bool& emit, int& nfold) {
-  const int kprev = __shfl_up_sync(kFull, key, 1);
-  const unsigned H = __ballot_sync(kFull, lane == 0 || kprev != key);
-  const int runstart = 31 - __clz(H & lanemask_le());
-  const unsigned later = H & ~lanemask_le();
-  const int runend = later ? __ffs(later) - 1 : 32;
-  emit = ((lane - runstart) % OMERF_FOLD) == 0;
-  nfold = emit ? min(OMERF_FOLD, runend - lane) : 0;  // lanes [lane, lane + nfold) share the stencil
+// Gradient scatter of a queue's 32 samples.  Four neighbouring lanes (samples
+// of a ray, mostly) take their four samples one after the other: lane j holds
+// channels 4 (j & 1) .. + 3 of the lower or upper (j >> 1) texel of every row,
+// a row being the two texels that are neighbours along the arrays' fast axis.
+// One instruction then reduces the 64 contiguous bytes of a row, and a run of
+// samples that share a cell or a plane footprint is summed in registers and
+// reduced once.  The L1 pipe bound the march when every emitting lane reduced
+// its own texels (85 % busy, 19 x 16-byte reductions per sample, each lane a
+// wavefront of its own); with 64-byte rows it is 48 % busy and the chain of
+// one queue's steps bounds it.  2^18 rays (field) 866 -> 839 us, 2^20 rays
+// (city) FP32 7.33 -> 6.89, BF16 6.52 -> 6.27 ms per step.  (Staging the rows
+// in shared memory instead of shuffling took 0.97 and 7.95 ms.)
+struct QuadDt {
+  float v[4][4];  // [sample of the quad][channel of this lane's half]
+};
+
+__device__ __forceinline__ void quad_exchange(const float dt[8], int lane, QuadDt& q) {
+  const bool hi = lane & 1;
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const float a = __shfl_sync(kFull, dt[c], i, 4), b = __shfl_sync(kFull, dt[4 + c], i, 4);
+      q.v[i][c] = hi ? b : a;
+    }
 }
 
-__device__ __forceinline__ void red8(float* base, int off, const float v[8]) {
-  float4* q = reinterpret_cast<float4*>(base + off);
-  atomicAdd(q, make_float4(v[0], v[1], v[2], v[3]));
-  atomicAdd(q + 1, make_float4(v[4], v[5], v[6], v[7]));
+// Bit l: lane l's sample is active and the next lane of its quad does not
+// continue its run of equal keys.
+__device__ __forceinline__ unsigned run_ends(int key, bool act, int lane) {
+  const int next = __shfl_down_sync(kFull, key, 1);
+  return __ballot_sync(kFull, act && ((lane & 3) == 3 || next != key));
+}
+
+__device__ __forceinline__ void red4(float* p, const float v[4]) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(v[0]),
+               "f"(v[1]), "f"(v[2]), "f"(v[3])
+               : "memory");
+}
+
+// The 4 rows (dx, dy) of the grid cell; off[8] and f[3] are this lane's sample's.
+__device__ __forceinline__ void scatter_grid(const Geo& g, float* __restrict__ buf, const int off[8], const float f[3],
+                                             const QuadDt& q, bool act, int lane) {
+  const unsigned ends = run_ends(act && off[0] >= 0 ? off[0] : -1 - lane, act, lane) >> (lane & 28);
+  const bool up = (lane >> 1) & 1;
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const float fx = __shfl_sync(kFull, f[0], i, 4), fy = __shfl_sync(kFull, f[1], i, 4),
+                fz = __shfl_sync(kFull, f[2], i, 4);
+    const float wz = up ? fz : 1.0f - fz;
+    const bool first = i == 0 || ((ends >> (i - 1)) & 1u), last = (ends >> i) & 1u;
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+      const int lo = __shfl_sync(kFull, off[2 * r], i, 4), hi = __shfl_sync(kFull, off[2 * r + 1], i, 4);
+      const float w = ((r & 2) ? fx : 1.0f - fx) * ((r & 1) ? fy : 1.0f - fy) * wz;
+#pragma unroll
+      for (int c = 0; c < 4; c++) acc[r][c] = fmaf(w, q.v[i][c], first ? 0.0f : acc[r][c]);
+      const int o = up ? hi : lo;
+      if (last && o >= 0 && in_range(g, 0, o)) red4(buf + o + 4 * (lane & 1), acc[r]);
+    }
+  }
+}
+
+// The 2 rows of a plane footprint: base texel `base`, row stride `su` elements.
+__device__ __forceinline__ void scatter_plane(const Geo& g, int array, float* __restrict__ buf, int base, int su,
+                                              float fu, float fv, const QuadDt& q, bool act, int lane) {
+  const unsigned ends = run_ends(act ? base : -1 - lane, act, lane) >> (lane & 28);
+  const bool up = (lane >> 1) & 1;
+  float acc[2][4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const float u = __shfl_sync(kFull, fu, i, 4), v = __shfl_sync(kFull, fv, i, 4);
+    const int o = __shfl_sync(kFull, base, i, 4) + (up ? kNch : 0);
+    const float wv = up ? v : 1.0f - v;
+    const bool first = i == 0 || ((ends >> (i - 1)) & 1u), last = (ends >> i) & 1u;
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+      const float w = (r ? u : 1.0f - u) * wv;
+#pragma unroll
+      for (int c = 0; c < 4; c++) acc[r][c] = fmaf(w, q.v[i][c], first ? 0.0f : acc[r][c]);
+      if (last && in_range(g, array, o + r * su)) red4(buf + o + r * su + 4 * (lane & 1), acc[r]);
+    }
+  }
 }
 
 // Per-warp shared state of the packed backward re-march of 32 rays.
@@ -478,10 +541,11 @@ __device__ __forceinline__ void march_bundle_bwd(const Geo& g, const BwdArgs& a,
     s.branch = 0;
 #pragma unroll
     for (int c = 0; c < 7; c++) s.x[c] = 0.0f;
-    int goff[8], poff[12];
-    float gw[8], pw[12];
+    int goff[8];
     if (act) {
       const float p[3] = {qa.x, qa.y, qa.z};
+      int poff[12];
+      float gw[8], pw[12];
       grid_stencil<SPARSE>(g, p, goff, gw);
       plane_stencil(g, p, poff, pw);
       float t[8];
@@ -527,55 +591,24 @@ __device__ __forceinline__ void march_bundle_bwd(const Geo& g, const BwdArgs& a,
       }
     }
     // gradient scatter (all lanes; inactive lanes contribute nothing)
-    // neighbours' dL/dt and weights, lanes +1 .. +OMERF_FOLD-1
-    float dtn[OMERF_FOLD - 1][8];
-#pragma unroll
-    for (int j = 1; j < OMERF_FOLD; j++)
-#pragma unroll
-      for (int c = 0; c < 8; c++) dtn[j - 1][c] = __shfl_down_sync(kFull, dt[c], j);
+    QuadDt q;
+    quad_exchange(dt, lane, q);
+    int pi[3];
+    float pf[3];
+    const float p[3] = {qa.x, qa.y, qa.z};
     if (a.g_grid) {
-      bool emit;
-      int nfold;
-      pair_fold_info(act && goff[0] >= 0 ? goff[0] : -1 - lane, lane, emit, nfold);
 #pragma unroll
-      for (int c = 0; c < 8; c++) {
-        float v[8];
-#pragma unroll
-        for (int ch = 0; ch < 8; ch++) v[ch] = gw[c] * dt[ch];
-#pragma unroll
-        for (int j = 1; j < OMERF_FOLD; j++) {
-          const float wn = __shfl_down_sync(kFull, gw[c], j);
-          if (j < nfold)
-#pragma unroll
-            for (int ch = 0; ch < 8; ch++) v[ch] = fmaf(wn, dtn[j - 1][ch], v[ch]);
-        }
-        if (act && emit && goff[c] >= 0 && in_range(g, 0, goff[c])) red8(a.g_grid, goff[c], v);
-      }
+      for (int c = 0; c < 3; c++) axis_coord(p[c], g.lo[c], g.gs[c], g.L[c], pi[c], pf[c]);
+      scatter_grid(g, a.g_grid, goff, pf, q, act, lane);
     }
-    {
-      float* gp[3] = {a.g_xy, a.g_xz, a.g_yz};
 #pragma unroll
-      for (int q = 0; q < 3; q++) {
-        if (!gp[q]) continue;
-        bool emit;
-        int nfold;
-        pair_fold_info(act ? poff[4 * q] : -1 - lane, lane, emit, nfold);
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-          float v[8];
-#pragma unroll
-          for (int ch = 0; ch < 8; ch++) v[ch] = pw[4 * q + c] * dt[ch];
-#pragma unroll
-          for (int j = 1; j < OMERF_FOLD; j++) {
-            const float wn = __shfl_down_sync(kFull, pw[4 * q + c], j);
-            if (j < nfold)
-#pragma unroll
-              for (int ch = 0; ch < 8; ch++) v[ch] = fmaf(wn, dtn[j - 1][ch], v[ch]);
-          }
-          if (act && emit && in_range(g, 1 + q, poff[4 * q + c])) red8(gp[q], poff[4 * q + c], v);
-        }
-      }
-    }
+    for (int c = 0; c < 3; c++) axis_coord(p[c], g.lo[c], g.ps[c], g.R[c], pi[c], pf[c], c == 2 ? g.pzoff : 0.0f);
+    if (a.g_xy)
+      scatter_plane(g, 1, a.g_xy, (pi[0] * g.R[1] + pi[1]) * kNch, g.R[1] * kNch, pf[0], pf[1], q, act, lane);
+    if (a.g_xz)
+      scatter_plane(g, 2, a.g_xz, (pi[0] * g.R[2] + pi[2]) * kNch, g.R[2] * kNch, pf[0], pf[2], q, act, lane);
+    if (a.g_yz)
+      scatter_plane(g, 3, a.g_yz, (pi[1] * g.R[2] + pi[2]) * kNch, g.R[2] * kNch, pf[1], pf[2], q, act, lane);
     const int rnext = __shfl_down_sync(kFull, r, 1);
     const bool tail = act && (lane == 31 || rnext != r);
     __syncwarp();
@@ -1156,13 +1189,15 @@ __global__ void __launch_bounds__(128, 1) mlp_bwd_tc_kernel(const Geo g, const B
 
 // Kernel 2: re-march every ray (one warp per bundle of 32 rays, persistent)
 // and scatter the per-sample gradients.
-#ifndef OMERF_BWD_MINB
-#define OMERF_BWD_MINB 2  // resident CTAs per SM the register budget is sized for
-#endif
+// CTAs of 4 warps, 5 per SM (96 registers): the warps take bundles on their
+// own, so small CTAs only set the register granularity.  City step (2^20 rays,
+// FP32 / BF16 features) with 4, 5, 6 CTAs per SM: 7.12 / 6.44, 6.89 / 6.27,
+// 7.52 / 6.84 ms (6 spills).
+constexpr int kMarchThreads = 128;
 
 template <class FT, bool SPARSE>
-__global__ void __launch_bounds__(kThreads, OMERF_BWD_MINB) march_bwd_kernel(const Geo g, const BwdArgs a) {
-  __shared__ WarpBwd sBwd[kThreads / 32];
+__global__ void __launch_bounds__(kMarchThreads, 5) march_bwd_kernel(const Geo g, const BwdArgs a) {
+  __shared__ WarpBwd sBwd[kMarchThreads / 32];
   const int lane = threadIdx.x & 31;
   WarpBwd& ws = sBwd[threadIdx.x >> 5];
   for (;;) {
@@ -1209,13 +1244,13 @@ static cudaError_t launch_bwd_variant(const omerf_scene* s, const BwdArgs& a, cu
   const int dev = s->device & 63;
   int nb = blocks[dev].load(std::memory_order_relaxed);
   if (nb == 0) {
-    nb = persistent_blocks((const void*)kern, kThreads, 0, s->num_sms);
+    nb = persistent_blocks((const void*)kern, kMarchThreads, 0, s->num_sms);
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
-  long want = (a.n_bundles + (kThreads / 32) - 1) / (kThreads / 32);
+  long want = (a.n_bundles + (kMarchThreads / 32) - 1) / (kMarchThreads / 32);
   int grid = (int)(want < nb ? want : nb);
   if (grid < 1) grid = 1;
-  kern<<<grid, kThreads, 0, stream>>>(s->geo, a);
+  kern<<<grid, kMarchThreads, 0, stream>>>(s->geo, a);
   return cudaGetLastError();
 }
 
