@@ -1,4 +1,5 @@
-// march_cam.cu -- FP32 camera render, a fixed set of lanes per ray (sm_103a).
+// march_cam.cu -- FP32 render with a fixed set of lanes per ray: cameras and
+// short ray lists (sm_103a).
 //
 // The L1 data pipe bounds the render: a 256-bit texel load takes one
 // wavefront per distinct 128-byte line in each group of four lanes, 20 loads
@@ -42,15 +43,15 @@ template <int G>
 struct CamShape;
 template <>
 struct CamShape<1> {
-  static constexpr int kWarps = 4, kW = 16, kH = 8;
+  static constexpr int kWarps = 4, kW = 16, kH = 8, kRays = kW * kH;
 };
 template <>
 struct CamShape<4> {
-  static constexpr int kWarps = 4, kW = 8, kH = 4;
+  static constexpr int kWarps = 4, kW = 8, kH = 4, kRays = kW * kH;
 };
 template <>
 struct CamShape<8> {
-  static constexpr int kWarps = 4, kW = 4, kH = 4;
+  static constexpr int kWarps = 4, kW = 4, kH = 4, kRays = kW * kH;
 };
 
 // Pixel of a lane's ray inside the super-tile.
@@ -171,23 +172,42 @@ __device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb,
   return *cam;
 }
 
-// March one 8 x 4 tile with the packed queue (32 rays of one warp) and write
-// the sample counts of the pixels whose bit is set in `want` (bit 8 y + x).
+__device__ __forceinline__ void load_ray(const float* __restrict__ r, float o[3], float d[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    o[c] = __ldg(r + c);
+    d[c] = __ldg(r + 3 + c);
+  }
+}
+
+// March the 32 rays of one of the packed queue's bundles (an 8 x 4 tile, bit
+// 8 y + x, or 32 consecutive rays of a list) with the queue, and write the
+// sample counts of the rays whose bit is set in `want`.
 template <class FT, bool SPARSE, int G>
-__device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, WarpMarch<false>& ws, unsigned sb, int tx,
-                                            int ty, unsigned want) {
+__device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, WarpMarch<false>& ws, unsigned sb, int t,
+                                            unsigned want) {
   const int lane = threadIdx.x & 31;
-  int x0, y0;
-  long ray0;
-  const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
-  const int px = ((x0 >> 3) + tx) * 8 + (lane & 7), py = ((y0 >> 2) + ty) * 4 + (lane >> 3);
-  const bool valid = px < cam.width && py < cam.height;
+  bool valid;
+  long rid;
   float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
-  if (valid) camera_ray(cam, px, py, o, d);
+  if (a.use_cam) {
+    constexpr int kTilesX = (CamShape<G>::kW + 7) / 8;
+    int x0, y0;
+    long ray0;
+    const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
+    const int px = ((x0 >> 3) + t % kTilesX) * 8 + (lane & 7), py = ((y0 >> 2) + t / kTilesX) * 4 + (lane >> 3);
+    valid = px < cam.width && py < cam.height;
+    rid = ray0 + (long)py * cam.width + px;
+    if (valid) camera_ray(cam, px, py, o, d);
+  } else {
+    rid = ((long)sb * CamShape<G>::kRays & ~31l) + 32 * t + lane;
+    valid = rid < a.n;
+    if (valid) load_ray(a.rays + 6 * rid, o, d);
+  }
   int klo = 0, khi = -1;
   const bool any = valid && lattice_range(g, o, d, klo, khi);
   march_bundle<FT, SPARSE>(g, lane, o, d, klo, khi, any, ws);
-  if (valid && ((want >> lane) & 1u)) a.count[ray0 + (long)py * cam.width + px] = ws.s.cnt[lane];
+  if (valid && ((want >> lane) & 1u)) a.count[rid] = ws.s.cnt[lane];
 }
 
 // 7 CTAs of 4 warps (72 registers) per SM: 2.91 ms per 1080p frame, 2.90 with
@@ -213,15 +233,29 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
     if (sb >= a.n_super) break;
     if (threadIdx.x == 0) sWork[it ^ 1] = atomicAdd(a.counter, 1u);
 
-    int sx, sy, x0, y0;
-    long ray0;
-    lane_pixel<G>(warp, lane, sx, sy);
+    bool valid;
+    long rid;
+    int amb_tile, amb_bit;  // the queue's bundle within the super-tile that holds this ray
     float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
-    const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
-    const int px = x0 + sx, py = y0 + sy;
-    const bool valid = px < cam.width && py < cam.height;
-    const long rid = ray0 + (long)py * cam.width + px;
-    if (valid) camera_ray(cam, px, py, o, d);
+    if (a.use_cam) {
+      int sx, sy, x0, y0;
+      long ray0;
+      lane_pixel<G>(warp, lane, sx, sy);
+      const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
+      const int px = x0 + sx, py = y0 + sy;
+      valid = px < cam.width && py < cam.height;
+      rid = ray0 + (long)py * cam.width + px;
+      if (valid) camera_ray(cam, px, py, o, d);
+      amb_tile = (sy / 4) * kTilesX + sx / 8;
+      amb_bit = ((py & 3) << 3) | (px & 7);
+    } else {
+      const int r = warp * (32 / G) + lane / G;
+      rid = (long)sb * CamShape<G>::kRays + r;
+      valid = rid < a.n;
+      if (valid) load_ray(a.rays + 6 * rid, o, d);
+      amb_tile = r >> 5;
+      amb_bit = (int)(rid & 31);
+    }
     int klo = 0, khi = -1;
     bool alive = valid && lattice_range(g, o, d, klo, khi);
     if (!alive) {
@@ -394,10 +428,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
       }
     }
     if constexpr (COUNT) {
-      if (amb && valid) {
-        const int tx = (x0 + sx) / 8 - x0 / 8, ty = (y0 + sy) / 4 - y0 / 4;
-        atomicOr(&sAmb[ty * kTilesX + tx], 1u << (((py & 3) << 3) | (px & 7)));
-      }
+      if (amb && valid) atomicOr(&sAmb[amb_tile], 1u << amb_bit);
       __syncthreads();
       if (warp == 0) {
         // rays whose transmittance passed the termination threshold within
@@ -406,7 +437,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
         for (int t = 0; t < kTilesX * kTilesY; t++) {
           const unsigned want = sAmb[t];
           if (want) {
-            resolve_counts<FT, SPARSE, G>(g, a, sMarch, sb, t % kTilesX, t / kTilesX, want);
+            resolve_counts<FT, SPARSE, G>(g, a, sMarch, sb, t, want);
             __syncwarp();
             if (lane == 0) sAmb[t] = 0u;
           }
@@ -448,6 +479,15 @@ static cudaError_t launch_cam_group(const omerf_scene* s, const FwdArgs& a, cuda
 int cam_lanes(const omerf_scene* s, long n) {
   if (s->desc.feat_dtype != OMERF_F32) return 0;
   return n < (1 << 17) ? 8 : (n < (1 << 20) ? 4 : 1);
+}
+
+// Rays of a list may lie anywhere: rays of different lengths share a warp, and
+// the queue, which packs samples whatever their ray, keeps its lanes busy.  Few
+// rays leave the chip idle, and there 8 lanes per ray shorten the chain (us
+// with the queue / 8 lanes, random city rays with counts: 3,001 rays 253 /
+// 180, 10,007 rays 256 / 176, 30,011 rays 259 / 276, 100,003 rays 319 / 693).
+int list_lanes(const omerf_scene* s, long n) {
+  return s->desc.feat_dtype == OMERF_F32 && n < (1 << 14) ? 8 : 0;
 }
 
 void cam_super(int lanes, int& w, int& h) {

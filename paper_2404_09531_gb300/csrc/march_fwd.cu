@@ -249,7 +249,10 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
     a.n_super = (long)a.super_x * ((cam->height + sh - 1) / sh);
   } else {
     a.use_cam = 0;
-    a.n_super = (n + 255) / 256;
+    lanes = train ? 0 : list_lanes(s, n);
+    int sw, sh;
+    cam_super(lanes, sw, sh);
+    a.n_super = (n + sw * sh - 1) / (sw * sh);
   }
   a.rays = rays;
   a.n = n;

@@ -37,3 +37,25 @@ def test_every_form_gives_the_same_pixels(cfg, size):
         p_rgb, _ = om.render_cameras(scene, [cam, fill], want_count=False)
         assert torch.equal(p_rgb[:n], rgb)
         assert torch.equal(p_rgb[n:], g_rgb[:-n])
+
+
+@pytest.mark.parametrize("cfg", [1, 2])
+@pytest.mark.parametrize("n", [1, 17, 1000, 16383])
+def test_short_ray_lists_match_long_ones(cfg, n):
+    """Fewer than 2^14 rays take 8 lanes each, more the packed queue: the same
+    counts, and pixels within the rounding of the two orders of summation."""
+    sc = synth.make_scene(cfg)
+    table, pool = brick_inputs(sc) if sc["spec"].brick else (None, None)
+    scene = gpu_scene(sc, table=table)
+    rays = torch.as_tensor(synth.make_train_batch(cfg, 16384, K=1)["rays"]).cuda()
+    long_rgb, long_cnt = om.render(scene, rays=rays)
+    rgb, cnt = om.render(scene, rays=rays[:n].contiguous())
+    only_rgb, _ = om.render(scene, rays=rays[:n].contiguous(), want_count=False)
+    assert torch.equal(cnt, long_cnt[:n])
+    assert torch.equal(only_rgb, rgb)
+    # about 50 sums of values below 1, each rounded by 2^-24, in either order
+    assert (rgb - long_rgb[:n]).abs().max().item() <= 2 * 50 * 2.0 ** -24
+    idx = np.arange(0, n, max(1, n // 500))
+    r = rays[:n].cpu().numpy()[idx]
+    ref = oracle.render(oracle_scene_for(sc, table, pool), r)
+    compare_render(rgb.cpu().numpy()[idx], cnt.cpu().numpy()[idx], ref, what=f"config {cfg}, {n} rays")
