@@ -11,6 +11,7 @@
 //                    allocates, from a dense grid or an older pool Sec. 4.4
 //   plane crop       the XZ / YZ plane rows that any evaluated sample can
 //                    reach, from the occupancy bounds              Sec. 4.4
+#include <algorithm>
 #include <cmath>
 
 #include <cuda.h>
@@ -20,40 +21,119 @@
 
 namespace omerf {
 
-// One thread per (i, j, 32-voxel word along z).  Bit b of word w is voxel
-// k = 32 w + b.  The z edges are FP32 without fused operations, as in the
-// definition; cell ranges are exact integer arithmetic.
-__global__ void __launch_bounds__(256) occupancy_grid_kernel(const float2* __restrict__ occ, int M, int Nx, int Ny,
-                                                            int Nz, float z0, float hz, uint32_t* __restrict__ bits,
-                                                            unsigned long long* count) {
-  const int W = (Nz + 31) >> 5;
-  const long long total = (long long)Nx * Ny * W;
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned pop = 0;
-  if (id < total) {
-    const int w = (int)(id % W);
-    const long long ij = id / W;
-    const int j = (int)(ij % Ny), i = (int)(ij / Ny);
-    const int alo = (int)((long long)i * M / Nx), ahi = (int)(((long long)(i + 1) * M + Nx - 1) / Nx) - 1;
-    const int blo = (int)((long long)j * M / Ny), bhi = (int)(((long long)(j + 1) * M + Ny - 1) / Ny) - 1;
-    const int k0 = 32 * w, nk = min(32, Nz - k0);
-    uint32_t word = 0;
-    for (int a = alo; a <= ahi; a++)
-      for (int b = blo; b <= bhi; b++) {
-        const float2 z = __ldg(occ + (long long)a * M + b);
-        if (!(z.x < z.y)) continue;
-        for (int t = 0; t < nk; t++) {
-          const float zl = __fadd_rn(z0, __fmul_rn((float)(k0 + t), hz));
-          const float zh = __fadd_rn(z0, __fmul_rn((float)(k0 + t + 1), hz));
-          if (z.x < zh && z.y > zl) word |= 1u << t;
-        }
-      }
-    bits[id] = word;
-    pop = __popc(word);
+// Voxel k of a column of voxels overlaps the interval (z.x, z.y) iff
+// z.x < zh(k) and z.y > zl(k), zl(k) = z0 + k hz and zh(k) = zl(k + 1) in FP32
+// without fused operations, as in the definition.  zl does not decrease with
+// k, so the voxels are those in [first, last]: the first k with zl(k + 1) > z.x
+// and the last with zl(k) < z.y.
+__device__ __forceinline__ float voxel_edge(float z0, float hz, int k) {
+  return __fadd_rn(z0, __fmul_rn((float)k, hz));
+}
+// The number of k in [0, n) with zl(k + SHIFT) below z (EQUAL: or at z): an
+// estimate that the edges on both sides confirm, else bisection.
+template <int SHIFT, bool EQUAL>
+__device__ __forceinline__ int edges_below(float z0, float hz, int n, float z) {
+  auto below = [&](int k) {
+    const float e = voxel_edge(z0, hz, k + SHIFT);
+    return EQUAL ? e <= z : e < z;
+  };
+  const float q = __fdividef(z - z0, hz);
+  const int guess = (int)fminf(fmaxf(q, 0.0f), (float)n) + 1 - SHIFT;  // (a NaN counts as 0)
+#pragma unroll
+  for (int t = 0; t < 2; t++) {
+    const int c = min(max(guess - t, 0), n);
+    if ((c == 0 || below(c - 1)) && (c == n || !below(c))) return c;
   }
-  if (count) {
-    for (int s = 16; s > 0; s >>= 1) pop += __shfl_xor_sync(kFull, pop, s);
-    if ((threadIdx.x & 31) == 0 && pop) atomicAdd(count, (unsigned long long)pop);
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (below(mid)) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+// first and last voxel of a column that overlap the interval z (first > last: none)
+__device__ __forceinline__ void voxel_range(float z0, float hz, int n, float2 z, int& first, int& last) {
+  first = edges_below<1, true>(z0, hz, n, z.x);
+  last = edges_below<0, false>(z0, hz, n, z.y) - 1;
+}
+// bits of voxels [first, last] in word w
+__device__ __forceinline__ uint32_t range_word(int first, int last, int w) {
+  const int lo = max(first - 32 * w, 0), hi = min(last - 32 * w, 31);
+  return lo > hi ? 0u : (~0u << lo) & (~0u >> (31 - hi));
+}
+
+// A warp takes 32 columns (i, j .. j + 31), one per lane, and writes their W =
+// ceil(Nz / 32) words in order (bit b of word w is voxel k = 32 w + b).  A
+// column that lies in one occupancy cell, the common case, has one interval,
+// found once; the words of a column that overlaps several cells are united
+// cell by cell.  Cell ranges are exact integer arithmetic, in 32 bits where
+// they fit (small).  Each block adds its voxel count once: an addition per
+// warp and word made the 16.8 M words of a 2048^2 x 128 grid queue for one
+// address (199 us, now 64 us; integer instructions bound it).
+__global__ void __launch_bounds__(256) occupancy_grid_kernel(const float2* __restrict__ occ, int M, int Nx, int Ny,
+                                                            int Nz, float z0, float hz, int small,
+                                                            uint32_t* __restrict__ bits, unsigned long long* count) {
+  __shared__ unsigned long long part[8];
+  const int W = (Nz + 31) >> 5, lane = threadIdx.x & 31;
+  const unsigned groups = ((unsigned)Ny + 31u) >> 5;  // of 32 columns in a row
+  const long long units = (long long)Nx * groups;
+  // cells [lo, hi] that voxel v of N along an axis overlaps
+  auto cells = [&](int v, int N, int& lo, int& hi) {
+    if (small) {
+      const unsigned a = (unsigned)v * (unsigned)M;
+      lo = (int)(a / (unsigned)N);
+      hi = (int)((a + (unsigned)M + (unsigned)N - 1u) / (unsigned)N) - 1;
+    } else {
+      lo = (int)((long long)v * M / N);
+      hi = (int)(((long long)(v + 1) * M + N - 1) / N) - 1;
+    }
+  };
+  unsigned long long pop = 0;
+  for (long long u = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); u < units; u += (long long)gridDim.x * 8) {
+    const int i = small ? (int)((unsigned)u / groups) : (int)(u / groups);
+    const int j0 = 32 * (int)(u - (long long)i * groups), j = j0 + lane;
+    int first = 1, last = 0, alo, ahi, blo = 0, bhi = -1;
+    cells(i, Nx, alo, ahi);
+    if (j < Ny) {
+      cells(j, Ny, blo, bhi);
+      if (alo == ahi && blo == bhi) {
+        const float2 z = __ldg(occ + (long long)alo * M + blo);
+        if (z.x < z.y) voxel_range(z0, hz, Nz, z, first, last);
+      }
+    }
+    const bool several = __any_sync(kFull, blo <= bhi && (alo < ahi || blo < bhi));
+    const int words = min(32, Ny - j0) * W;
+    uint32_t* out = bits + ((long long)i * Ny + j0) * W;
+    for (int e0 = 0; e0 < words; e0 += 32) {
+      const int e = e0 + lane, col = min(e / W, 31), w = e - col * W;
+      const int f = __shfl_sync(kFull, first, col), l = __shfl_sync(kFull, last, col);
+      uint32_t word = range_word(f, l, w);
+      if (several) {
+        const int b0 = __shfl_sync(kFull, blo, col), b1 = __shfl_sync(kFull, bhi, col);
+        if (e < words && (alo < ahi || b0 < b1))
+          for (int a = alo; a <= ahi; a++)
+            for (int b = b0; b <= b1; b++) {
+              const float2 z = __ldg(occ + (long long)a * M + b);
+              int zf, zl;
+              if (!(z.x < z.y)) continue;
+              voxel_range(z0, hz, Nz, z, zf, zl);
+              word |= range_word(zf, zl, w);
+            }
+      }
+      if (e < words) {
+        out[e] = word;
+        pop += __popc(word);
+      }
+    }
+  }
+  if (!count) return;
+  for (int s = 16; s > 0; s >>= 1) pop += __shfl_xor_sync(kFull, pop, s);
+  if (lane == 0) part[threadIdx.x >> 5] = pop;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) pop += part[w];
+    if (pop) atomicAdd(count, pop);
   }
 }
 
@@ -173,16 +253,25 @@ __global__ void __launch_bounds__(32) extract_bricks_tma_kernel(const __grid_con
 
 // Hull of the non-empty cells (z_min < z_max strictly: a sample needs
 // z_min < z < z_max) and the crop rule, in one block.
-__global__ void plane_crop_kernel(const float2* __restrict__ occ, long long cells, float pz0, float pz1, int Rz,
-                                  int* __restrict__ rows, float* __restrict__ zr) {
+// (eight rounds of loads in flight, as in hull_kernel)
+__global__ void __launch_bounds__(1024) plane_crop_kernel(const float2* __restrict__ occ, long long cells, float pz0,
+                                                          float pz1, int Rz, int* __restrict__ rows,
+                                                          float* __restrict__ zr) {
   __shared__ float slo[32], shi[32];
   float lo = __int_as_float(0x7f800000), hi = -lo;
-  for (long long c = threadIdx.x; c < cells; c += blockDim.x) {
-    const float2 z = occ[c];
-    if (z.x < z.y) {
-      lo = fminf(lo, z.x);
-      hi = fmaxf(hi, z.y);
+  for (long long c0 = threadIdx.x; c0 < cells; c0 += 8 * blockDim.x) {
+    float2 z[8];
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+      const long long c = c0 + r * (long long)blockDim.x;
+      z[r] = c < cells ? __ldg(occ + c) : make_float2(1.0f, -1.0f);
     }
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+      if (z[r].x < z[r].y) {
+        lo = fminf(lo, z[r].x);
+        hi = fmaxf(hi, z[r].y);
+      }
   }
   for (int s = 16; s > 0; s >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(kFull, lo, s));
@@ -285,13 +374,14 @@ omerf_status omerf_occupancy_grid(const float aabb[6], const float* occ, int32_t
   const long long words = (long long)N[0] * N[1] * ((N[2] + 31) / 32);
   if (words > (1LL << 40)) { set_error("occupancy grid too large"); return OMERF_ESHAPE; }
   const float hz = (aabb[5] - aabb[4]) / (float)N[2];
-  const long long blocks = (words + 255) / 256;
-  if (blocks > 0x7fffffffLL) { set_error("occupancy grid too large"); return OMERF_ESHAPE; }
+  if ((words + 255) / 256 > 0x7fffffffLL) { set_error("occupancy grid too large"); return OMERF_ESHAPE; }
   OMERF_LAUNCH_FAULT();
   omerf_status st = check_device_ptrs({{occ, "occ"}, {bits, "bits"}, {count, "count"}});
   if (st != OMERF_OK) return st;
-  occupancy_grid_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(
-      reinterpret_cast<const float2*>(occ), M, N[0], N[1], N[2], aabb[4], hz, bits, count);
+  const long long units = (long long)N[0] * ((N[1] + 31ll) / 32);
+  const int small = units < (1ll << 31) && ((long long)std::max(N[0], N[1]) + 1) * M + std::max(N[0], N[1]) < (1ll << 31);
+  occupancy_grid_kernel<<<grid_for(units, 8, 8 * sm_count()), 256, 0, (cudaStream_t)stream>>>(
+      reinterpret_cast<const float2*>(occ), M, N[0], N[1], N[2], aabb[4], hz, small, bits, count);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OMERF_OK : cuda_fail(e, "occupancy grid launch");
 }

@@ -34,15 +34,25 @@ unsigned* next_counter(const omerf_scene* s, cudaStream_t stream) {
 // ---------------------------------------------------------------------------
 // occupancy hull: min z_min and max z_max over the non-empty cells
 // ---------------------------------------------------------------------------
-__global__ void hull_kernel(const float2* __restrict__ occ, long cells, float* __restrict__ hull) {
+// One block (no second pass, no atomics): the loads of eight rounds are in
+// flight together (65,536 cells 10.0 us, 13.0 us one round at a time).
+__global__ void __launch_bounds__(1024) hull_kernel(const float2* __restrict__ occ, long cells,
+                                                    float* __restrict__ hull) {
   __shared__ float slo[32], shi[32];
   float lo = __int_as_float(0x7f800000), hi = -lo;
-  for (long i = threadIdx.x; i < cells; i += blockDim.x) {
-    float2 z = occ[i];
-    if (z.x <= z.y) {
-      lo = fminf(lo, z.x);
-      hi = fmaxf(hi, z.y);
+  for (long i0 = threadIdx.x; i0 < cells; i0 += 8 * blockDim.x) {
+    float2 z[8];
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+      const long i = i0 + r * (long)blockDim.x;
+      z[r] = i < cells ? __ldg(occ + i) : make_float2(1.0f, -1.0f);
     }
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+      if (z[r].x <= z[r].y) {
+        lo = fminf(lo, z[r].x);
+        hi = fmaxf(hi, z[r].y);
+      }
   }
   for (int s = 16; s > 0; s >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(kFull, lo, s));
@@ -164,29 +174,45 @@ __global__ void brick_table_check_kernel(const int* __restrict__ table, long tot
   if (b < -1 || b >= n_bricks) atomicAdd(bad, 1u);
 }
 
-// In-place exclusive scan of the 0/1 flags into pool indices (-1 = empty),
-// one CTA, each thread owning a contiguous segment (x-major brick order).
-__global__ void brick_scan_kernel(int* table, long total, int* n_alloc) {
-  __shared__ int sums[1024];
-  const long per = (total + blockDim.x - 1) / blockDim.x;
-  const long beg = threadIdx.x * per, end = beg + per < total ? beg + per : total;
-  int local = 0;
-  for (long i = beg; i < end; i++) local += table[i];
-  sums[threadIdx.x] = local;
-  __syncthreads();
-  for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-    int v = threadIdx.x >= (unsigned)off ? sums[threadIdx.x - off] : 0;
+// In-place exclusive scan of the 0/1 flags into pool indices (-1 = empty), one
+// CTA, x-major brick order.  A round scans 32 warps x 16 x 32 flags: a warp's
+// flags are 16 coalesced loads whose ballots are the scan within it (16,384
+// flags 9.6 us, 20 us with a contiguous segment per thread).
+__global__ void __launch_bounds__(1024) brick_scan_kernel(int* table, long total, int* n_alloc) {
+  constexpr int kRows = 16;
+  __shared__ int sums[2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int carry = 0, buf = 0;
+  for (long base = 0; base < total; base += 1024 * kRows, buf ^= 1) {
+    const long w0 = base + (long)warp * 32 * kRows + lane;
+    int f[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; r++) f[r] = w0 + 32 * r < total ? table[w0 + 32 * r] : 0;
+    int n = 0;
+    unsigned m[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      m[r] = __ballot_sync(kFull, f[r] != 0);
+      n += __popc(m[r]);
+    }
+    if (lane == 0) sums[buf][warp] = n;
     __syncthreads();
-    sums[threadIdx.x] += v;
-    __syncthreads();
+    // the warps' exclusive prefix: every warp scans the 32 counts itself
+    int v = sums[buf][lane], inc = v;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int u = __shfl_up_sync(kFull, inc, s);
+      if (lane >= s) inc += u;
+    }
+    int run = carry + __shfl_sync(kFull, inc - v, warp);
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      if (w0 + 32 * r < total) table[w0 + 32 * r] = f[r] ? run + __popc(m[r] & lanemask_lt()) : -1;
+      run += __popc(m[r]);
+    }
+    carry += __shfl_sync(kFull, inc, 31);
   }
-  int run = sums[threadIdx.x] - local;
-  for (long i = beg; i < end; i++) {
-    const int f = table[i];
-    table[i] = f ? run : -1;
-    run += f;
-  }
-  if (threadIdx.x == blockDim.x - 1) *n_alloc = sums[threadIdx.x];
+  if (threadIdx.x == 0) *n_alloc = carry;
 }
 
 // ---------------------------------------------------------------------------
