@@ -34,7 +34,9 @@ struct BwdArgs {
   const float* target;
   const float* dirs;
   int K;
-  long n, n_bundles;
+  int tiles;   // MLP backward: tiles of 16 rays per warp (1 or 2)
+  int bundle;  // re-march: rays per warp (up to 32)
+  long n, n_bundles;  // warps' units of either kernel
   float lam_rgb, lam_smooth;  // divided by n
   float* saved;
   const float* grad_scale;
@@ -149,11 +151,11 @@ __device__ __forceinline__ void zero_acc(DwAcc& acc) {
 
 // Add the warp's 32 staged rows (x 0..33, h1 34..49, h2 50..65, g1 66..81,
 // g2 82..97, g3 98..100) to the accumulators.  All 32 lanes must call it.
-__device__ __forceinline__ void accumulate_mma(const float* __restrict__ rows, int lane, DwAcc& acc) {
+__device__ __forceinline__ void accumulate_mma(const float* __restrict__ rows, int lane, int tiles, DwAcc& acc) {
   __syncwarp();
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll 1
-  for (int s = 0; s < 4; s++) {  // rays 8 s .. 8 s + 7 (the k dimension)
+  for (int s = 0; s < 2 * tiles; s++) {  // rays 8 s .. 8 s + 7 (the k dimension)
     const float* r0 = rows + (8 * s + t) * kRow;
     const float* r1 = rows + (8 * s + t + 4) * kRow;
     uint32_t ah[4], al[4];
@@ -230,11 +232,11 @@ __device__ __forceinline__ void store_acc(const DwAcc& acc, int lane, float* __r
 // G for the warp's 32 staged rows (x in columns 0..33): writes h1 (34..49),
 // h2 (50..65) and this lane's sigmoid outputs y.  All 32 lanes call it.
 __device__ __forceinline__ void warp_mlp_forward(float* __restrict__ rows, const MlpBwdShared& S, int lane,
-                                                 float y[3]) {
+                                                 int tiles, float y[3]) {
   __syncwarp();
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     float c[2][4];
@@ -264,7 +266,7 @@ __device__ __forceinline__ void warp_mlp_forward(float* __restrict__ rows, const
   }
   __syncwarp();
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     float c[2][4];
@@ -295,7 +297,7 @@ __device__ __forceinline__ void warp_mlp_forward(float* __restrict__ rows, const
   __syncwarp();
   // layer 3: B[k = unit2][n = output] = W3[output][unit2], outputs 0..2 of 8
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     float c[4];
@@ -329,7 +331,7 @@ __device__ __forceinline__ void warp_mlp_forward(float* __restrict__ rows, const
 // deltas g3 (98..100), g2 (82..97) and g1 (66..81).  A ReLU unit is active
 // iff its staged output is positive.  All 32 lanes call it.
 __device__ __forceinline__ void warp_mlp_backward(float* __restrict__ rows, const MlpBwdShared& S, int lane,
-                                                  const float y[3], const float gy[3]) {
+                                                  int tiles, const float y[3], const float gy[3]) {
   const int g = lane >> 2, t = lane & 3;
   {
     float* row = rows + lane * kRow;
@@ -339,7 +341,7 @@ __device__ __forceinline__ void warp_mlp_backward(float* __restrict__ rows, cons
   __syncwarp();
   // g2 = (G3 . W3) masked: K = 3 outputs (one k8 block, rows t < 3)
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     uint32_t ah[4], al[4];
@@ -359,7 +361,7 @@ __device__ __forceinline__ void warp_mlp_backward(float* __restrict__ rows, cons
   __syncwarp();
   // g1 = (G2 . W2) masked
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     float c[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
@@ -388,11 +390,11 @@ __device__ __forceinline__ void warp_mlp_backward(float* __restrict__ rows, cons
 // dL/dF = G1 . W1[:, :7] for the warp's rows, added into this lane's gF.
 // Uses the x columns 0..6 as scratch: call after the weight-gradient products.
 __device__ __forceinline__ void warp_mlp_input_grad(float* __restrict__ rows, const MlpBwdShared& S, int lane,
-                                                    float gF[7]) {
+                                                    int tiles, float gF[7]) {
   __syncwarp();
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll 1
-  for (int mt = 0; mt < 2; mt++) {
+  for (int mt = 0; mt < tiles; mt++) {
     float* r0 = rows + (16 * mt + g) * kRow;
     float* r1 = r0 + 8 * kRow;
     float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -634,13 +636,14 @@ __global__ void __launch_bounds__(kBwdThreads, 4) mlp_bwd_kernel(const Geo g, co
   __syncthreads();
   const float gs = a.grad_scale ? __ldg(a.grad_scale) : 1.0f;
   const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
+  const int tiles = a.tiles;
   const bool want_dw = a.g_mlp != nullptr;
   DwAcc acc;
   zero_acc(acc);
   float l_rgb = 0.0f, l_smooth = 0.0f;
   for (long b = (long)blockIdx.x * (blockDim.x >> 5) + warp; b < a.n_bundles; b += nwarps) {
-    const long rid = b * 32 + lane;
-    const bool valid = rid < a.n;
+    const long rid = b * 16 * tiles + lane;
+    const bool valid = lane < 16 * tiles && rid < a.n;
     float d[3] = {0, 0, 1};
     float F[7] = {0, 0, 0, 0, 0, 0, 0}, TN = 1.0f;
     int cnt = 0;
@@ -658,7 +661,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) mlp_bwd_kernel(const Geo g, co
     float gF[7] = {0, 0, 0, 0, 0, 0, 0};
     float gC[3] = {0, 0, 0}, yd[3] = {0, 0, 0}, gyd[3] = {0, 0, 0};
     stage_x(row, live, F, d);
-    warp_mlp_forward(rows, S, lane, yd);
+    warp_mlp_forward(rows, S, lane, tiles, yd);
     if (live) {
       float e[3], e2 = 0.0f;
 #pragma unroll
@@ -698,7 +701,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) mlp_bwd_kernel(const Geo g, co
       }
       stage_x(row, live, F, sh);
       float ys[3], gys[3] = {0.0f, 0.0f, 0.0f};
-      warp_mlp_forward(rows, S, lane, ys);
+      warp_mlp_forward(rows, S, lane, tiles, ys);
       if (live) {
         float q = 0.0f;
 #pragma unroll
@@ -709,17 +712,17 @@ __global__ void __launch_bounds__(kBwdThreads, 4) mlp_bwd_kernel(const Geo g, co
         }
         l_smooth = fmaf(S_cos, q, l_smooth);
       }
-      warp_mlp_backward(rows, S, lane, ys, gys);
-      if (want_dw) accumulate_mma(rows, lane, acc);
-      warp_mlp_input_grad(rows, S, lane, gF);
+      warp_mlp_backward(rows, S, lane, tiles, ys, gys);
+      if (want_dw) accumulate_mma(rows, lane, tiles, acc);
+      warp_mlp_input_grad(rows, S, lane, tiles, gF);
     }
     // the evaluation at d, recomputed (the smoothness evaluations reused the rows)
     float y[3];
     stage_x(row, live, F, d);
-    warp_mlp_forward(rows, S, lane, y);
-    warp_mlp_backward(rows, S, lane, y, gyd);
-    if (want_dw) accumulate_mma(rows, lane, acc);
-    warp_mlp_input_grad(rows, S, lane, gF);
+    warp_mlp_forward(rows, S, lane, tiles, y);
+    warp_mlp_backward(rows, S, lane, tiles, y, gyd);
+    if (want_dw) accumulate_mma(rows, lane, tiles, acc);
+    warp_mlp_input_grad(rows, S, lane, tiles, gF);
     if (valid) {
 #pragma unroll
       for (int j = 0; j < 3; j++) gF[j] += gC[j];
@@ -1200,13 +1203,16 @@ __global__ void __launch_bounds__(kMarchThreads, 5) march_bwd_kernel(const Geo g
   __shared__ WarpBwd sBwd[kMarchThreads / 32];
   const int lane = threadIdx.x & 31;
   WarpBwd& ws = sBwd[threadIdx.x >> 5];
-  for (;;) {
-    unsigned b = 0;
-    if (lane == 0) b = atomicAdd(a.counter, 1u);
-    b = __shfl_sync(kFull, b, 0);
+  for (bool first = true;; first = false) {
+    // without a counter there is one bundle per warp
+    unsigned b = first ? blockIdx.x * (kMarchThreads / 32) + (threadIdx.x >> 5) : (unsigned)a.n_bundles;
+    if (a.counter) {
+      if (lane == 0) b = atomicAdd(a.counter, 1u);
+      b = __shfl_sync(kFull, b, 0);
+    }
     if (b >= a.n_bundles) break;
-    const long rid = (long)b * 32 + lane;
-    const bool valid = rid < a.n;
+    const long rid = (long)b * a.bundle + lane;
+    const bool valid = lane < a.bundle && rid < a.n;
     float o[3] = {0, 0, 0}, d[3] = {0, 0, 1};
     int cnt = 0, klo = 0, khi = -1;
     if (valid) {
@@ -1247,10 +1253,18 @@ static cudaError_t launch_bwd_variant(const omerf_scene* s, const BwdArgs& a, cu
     nb = persistent_blocks((const void*)kern, kMarchThreads, 0, s->num_sms);
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
-  long want = (a.n_bundles + (kMarchThreads / 32) - 1) / (kMarchThreads / 32);
-  int grid = (int)(want < nb ? want : nb);
-  if (grid < 1) grid = 1;
-  kern<<<grid, kMarchThreads, 0, stream>>>(s->geo, a);
+  // Rays per warp: 32, fewer while that leaves warp slots of the chip empty
+  // (a warp's queue then spans fewer rays and its chain is shorter): 5,003
+  // rays (field) 116 -> 30 us with 4 rays per warp, 2^14 rays 123 -> 48 us.
+  BwdArgs b = a;
+  const long slots = (long)nb * (kMarchThreads / 32);
+  b.bundle = 32;
+  while (b.bundle > 4 && (a.n + b.bundle - 1) / b.bundle < slots) b.bundle /= 2;
+  b.n_bundles = (a.n + b.bundle - 1) / b.bundle;
+  const long want = (b.n_bundles + (kMarchThreads / 32) - 1) / (kMarchThreads / 32);
+  const int grid = (int)(want < nb ? want : nb);
+  b.counter = want <= grid ? nullptr : next_counter(s, stream);
+  kern<<<grid < 1 ? 1 : grid, kMarchThreads, 0, stream>>>(s->geo, b);
   return cudaGetLastError();
 }
 
@@ -1288,10 +1302,14 @@ static cudaError_t launch_mlp_bwd(const omerf_scene* s, const BwdArgs& a, cudaSt
     nb = persistent_blocks((const void*)mlp_bwd_kernel, kBwdThreads, smem, s->num_sms);
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
-  long want = (a.n_bundles + (kBwdThreads / 32) - 1) / (kBwdThreads / 32);
-  int grid = (int)(want < nb ? want : nb);
-  if (grid < 1) grid = 1;
-  mlp_bwd_kernel<<<grid, kBwdThreads, smem, stream>>>(s->geo, a);
+  // 32 rays per warp, 16 while that leaves warp slots of the chip empty (5,003
+  // rays, K = 3: 50 -> 45 us)
+  BwdArgs b = a;
+  b.tiles = (a.n + 31) / 32 < (long)nb * (kBwdThreads / 32) ? 1 : 2;
+  b.n_bundles = (a.n + 16 * b.tiles - 1) / (16 * b.tiles);
+  const long want = (b.n_bundles + (kBwdThreads / 32) - 1) / (kBwdThreads / 32);
+  const int grid = (int)(want < nb ? want : nb);
+  mlp_bwd_kernel<<<grid < 1 ? 1 : grid, kBwdThreads, smem, stream>>>(s->geo, b);
   return cudaGetLastError();
 }
 
@@ -1306,7 +1324,6 @@ cudaError_t launch_march_bwd(const omerf_scene* s, const float* rays, const floa
   a.dirs = dirs;
   a.K = K;
   a.n = n;
-  a.n_bundles = (n + 31) / 32;
   a.lam_rgb = n > 0 ? lam[0] / (float)n : 0.0f;
   a.lam_smooth = n > 0 ? lam[1] / (float)n : 0.0f;
   a.saved = saved;
@@ -1321,10 +1338,9 @@ cudaError_t launch_march_bwd(const omerf_scene* s, const float* rays, const floa
   // OMERF_FAULT=mlp_wait: the tcgen05 MLP backward's first wait gives up at
   // once (its products still complete and are waited for), for tests
   a.wait_tries = fault_injected("mlp_wait") ? 0 : tcmlp::kTries;
-  if (a.n_bundles == 0) return cudaSuccess;
+  if (n == 0) return cudaSuccess;
   cudaError_t e = launch_mlp_bwd(s, a, stream);
   if (e != cudaSuccess) return e;
-  a.counter = next_counter(s, stream);
   const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
   const bool sparse = s->desc.brick > 0;
   if (bf16) return sparse ? launch_bwd_variant<__nv_bfloat16, true>(s, a, stream)

@@ -215,7 +215,6 @@ __device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, Warp
 template <class FT, bool SPARSE, int G, bool COUNT>
 __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
     march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
-  constexpr int kWarps = CamShape<G>::kWarps;
   constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
   constexpr unsigned kFrameMask = (1u << kFrame) - 1u;
   constexpr int kTilesX = (CamShape<G>::kW + 7) / 8, kTilesY = (CamShape<G>::kH + 3) / 4;
@@ -226,12 +225,13 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
   if (COUNT && threadIdx.x < kTilesX * kTilesY) sAmb[threadIdx.x] = 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int base = lane & ~(kFrame - 1), j = G == 1 ? 0 : lane & (G - 1);
-  if (threadIdx.x == 0) sWork[0] = atomicAdd(a.counter, 1u);
+  // (without a counter there is one super-tile per CTA)
+  if (threadIdx.x == 0) sWork[0] = a.counter ? atomicAdd(a.counter, 1u) : blockIdx.x;
   __syncthreads();
   for (int it = 0;; it ^= 1) {
     const unsigned sb = sWork[it];
     if (sb >= a.n_super) break;
-    if (threadIdx.x == 0) sWork[it ^ 1] = atomicAdd(a.counter, 1u);
+    if (threadIdx.x == 0) sWork[it ^ 1] = a.counter ? atomicAdd(a.counter, 1u) : (unsigned)a.n_super;
 
     bool valid;
     long rid;
@@ -460,7 +460,9 @@ static cudaError_t launch_cam_variant(const omerf_scene* s, const FwdArgs& a, cu
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
   const int grid = (int)(a.n_super < nb ? a.n_super : nb);
-  kern<<<grid < 1 ? 1 : grid, threads, 0, stream>>>(s->geo, a);
+  FwdArgs b = a;
+  b.counter = a.n_super <= grid ? nullptr : next_counter(s, stream);
+  kern<<<grid < 1 ? 1 : grid, threads, 0, stream>>>(s->geo, b);
   return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
   __shared__ WarpMarch<kMMA> sMarch[kThreads / 32];
   if constexpr (kMMA) {
     build_mlp_frags(g.mlp, sFrag);
-  } else {
+  } else if constexpr (!TRAIN || LOSS) {
     load_mlp_padded(g.mlp, sW);
   }
   __syncthreads();
@@ -52,10 +52,12 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
   // The CTA takes work in units of 8 bundles so that its 8 warps march
   // neighbouring rays together and share L1 lines: a camera super-tile of
   // 2 x 4 tiles of 8 x 4 pixels (16 x 16 pixels), or 256 consecutive rays.
+  // Without a counter there is one unit per CTA.
   __shared__ unsigned sWork;
   const int warp = threadIdx.x >> 5;
-  for (;;) {
-    if (threadIdx.x == 0) sWork = atomicAdd(a.counter, 1u);
+  for (bool first = true;; first = false) {
+    if (threadIdx.x == 0)
+      sWork = a.counter ? atomicAdd(a.counter, 1u) : (first ? blockIdx.x : (unsigned)a.n_super);
     __syncthreads();
     const unsigned sb = sWork;
     __syncthreads();
@@ -226,10 +228,11 @@ static cudaError_t launch_variant(const omerf_scene* s, const FwdArgs& a, cudaSt
     nb = persistent_blocks((const void*)kern, kThreads, 0, s->num_sms);
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
-  long want = a.n_super;
-  int grid = (int)(want < nb ? want : nb);
-  if (grid < 1) grid = 1;
-  kern<<<grid, kThreads, 0, stream>>>(s->geo, a);
+  FwdArgs b = a;
+  const int grid = (int)(b.n_super < nb ? b.n_super : nb);
+  // as many CTAs as units: no work counter (and no launch to zero it)
+  b.counter = b.n_super <= grid ? nullptr : next_counter(s, stream);
+  kern<<<grid < 1 ? 1 : grid, kThreads, 0, stream>>>(s->geo, b);
   return cudaGetLastError();
 }
 
@@ -268,7 +271,6 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
   a.saved = saved;
   a.loss = loss;
   if (a.n_super == 0) return cudaSuccess;
-  a.counter = next_counter(s, stream);
   if (lanes > 0) return launch_render_cam(s, a, lanes, stream);
   const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
   const bool sparse = s->desc.brick > 0;
@@ -300,7 +302,6 @@ cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int 
   a.rgb = rgb;
   a.count = count;
   if (a.n_super == 0) return cudaSuccess;
-  a.counter = next_counter(s, stream);
   if (lanes > 0) return launch_render_cam(s, a, lanes, stream);
   const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
   const bool sparse = s->desc.brick > 0;
