@@ -525,9 +525,7 @@ struct WarpBwd {
 template <class FT, bool SPARSE>
 __device__ __forceinline__ void march_bundle_bwd(const Geo& g, const BwdArgs& a, int lane, const float o[3],
                                                  const float d[3], int klo, int khi, bool live, WarpBwd& ws) {
-  ws.q.ro[lane] = make_float4(o[0], o[1], o[2], __int_as_float(klo));
-  ws.q.rd[lane] = make_float4(d[0], d[1], d[2], __int_as_float(khi));
-  ws.q.cap[lane] = ws.cnt[lane];
+  queue_ray(g, ws.q, lane, o, d, klo, live ? khi : klo - 1, ws.cnt[lane]);
   unsigned pend = __ballot_sync(kFull, live);
   FillState f;
   __syncwarp();

@@ -51,9 +51,7 @@ __device__ __forceinline__ void march_bundle(const Geo& g, int lane, const float
   for (int c = 0; c < 8; c++) ws.s.F[lane][c] = 0.0f;
   ws.s.T[lane] = 1.0f;
   ws.s.cnt[lane] = 0;
-  ws.s.q.ro[lane] = make_float4(o[0], o[1], o[2], __int_as_float(klo));
-  ws.s.q.rd[lane] = make_float4(d[0], d[1], d[2], __int_as_float(khi));
-  ws.s.q.cap[lane] = g.n_max;
+  queue_ray(g, ws.s.q, lane, o, d, klo, any ? khi : klo - 1, g.n_max);
   unsigned pend = __ballot_sync(kFull, any);
   FillState f;
   __syncwarp();
