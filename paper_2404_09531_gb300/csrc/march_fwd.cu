@@ -1,9 +1,7 @@
 // march_fwd.cu -- forward march: render and training forward (sm_103a).
 //
-// Persistent kernel of 8 warps per CTA.  A CTA takes a super-tile of 8
-// bundles from an atomic work counter (16 x 16 pixels of a camera, or 256
-// consecutive rays of a ray list) so that its warps share L1 lines; a warp
-// owns a bundle of 32 rays (an 8 x 4 pixel tile).  The warp walks its rays
+// Persistent kernel of 8 warps per CTA; a warp owns a bundle of 32 rays at a
+// time (an 8 x 4 pixel tile of a camera, or 32 consecutive rays of a list).  The warp walks its rays
 // in order and packs their evaluated samples (Sec. 4.1: only samples inside
 // the occupancy interval are evaluated) into a 32-entry queue that may span
 // rays (packed.cuh); the 32 queued samples are gathered and activated in
@@ -49,18 +47,28 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
   WarpMarch<kMMA>& ws = sMarch[threadIdx.x >> 5];
   float l_rgb = 0.0f, l_smooth = 0.0f;
 
-  // The CTA takes work in units of 8 bundles so that its 8 warps march
-  // neighbouring rays together and share L1 lines: a camera super-tile of
-  // 2 x 4 tiles of 8 x 4 pixels (16 x 16 pixels), or 256 consecutive rays.
-  // Without a counter there is one unit per CTA.
+  // A camera: the CTA takes super-tiles of 2 x 4 tiles of 8 x 4 pixels (16 x
+  // 16 pixels), so that its 8 warps march neighbouring rays together and share
+  // L1 lines.  A list: every warp takes its next 32 consecutive rays on its
+  // own, without waiting for the CTA's slowest bundle (the rays of a training
+  // batch lie anywhere).  Without a counter there is one unit per CTA or warp.
   __shared__ unsigned sWork;
   const int warp = threadIdx.x >> 5;
   for (bool first = true;; first = false) {
-    if (threadIdx.x == 0)
-      sWork = a.counter ? atomicAdd(a.counter, 1u) : (first ? blockIdx.x : (unsigned)a.n_super);
-    __syncthreads();
-    const unsigned sb = sWork;
-    __syncthreads();
+    unsigned sb;
+    if (a.use_cam) {
+      if (threadIdx.x == 0)
+        sWork = a.counter ? atomicAdd(a.counter, 1u) : (first ? blockIdx.x : (unsigned)a.n_super);
+      __syncthreads();
+      sb = sWork;
+      __syncthreads();
+    } else {
+      sb = first ? blockIdx.x * (kThreads / 32) + warp : (unsigned)a.n_super;
+      if (a.counter) {
+        if (lane == 0) sb = atomicAdd(a.counter, 1u);
+        sb = __shfl_sync(kFull, sb, 0);
+      }
+    }
     if (sb >= a.n_super) break;
 
     long rid;
@@ -85,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
       rid = (long)py * a.cam.width + px;
       if (valid) camera_ray(a.cam, px, py, o, d);
     } else {
-      rid = ((long)sb * 8 + warp) * 32 + lane;
+      rid = (long)sb * 32 + lane;
       valid = rid < a.n;
       if (valid) {
         const float* r = a.rays + 6 * rid;
@@ -228,10 +236,12 @@ static cudaError_t launch_variant(const omerf_scene* s, const FwdArgs& a, cudaSt
     nb = persistent_blocks((const void*)kern, kThreads, 0, s->num_sms);
     blocks[dev].store(nb, std::memory_order_relaxed);
   }
+  // units: super-tiles of a camera, one CTA each; bundles of a list, one warp each
+  const long want = a.use_cam ? a.n_super : (a.n_super + kThreads / 32 - 1) / (kThreads / 32);
+  const int grid = (int)(want < nb ? want : nb);
   FwdArgs b = a;
-  const int grid = (int)(b.n_super < nb ? b.n_super : nb);
-  // as many CTAs as units: no work counter (and no launch to zero it)
-  b.counter = b.n_super <= grid ? nullptr : next_counter(s, stream);
+  // every unit has its CTA or warp: no work counter (and no launch to zero it)
+  b.counter = want <= grid ? nullptr : next_counter(s, stream);
   kern<<<grid < 1 ? 1 : grid, kThreads, 0, stream>>>(s->geo, b);
   return cudaGetLastError();
 }
@@ -253,8 +263,8 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
   } else {
     a.use_cam = 0;
     lanes = train ? 0 : list_lanes(s, n);
-    int sw, sh;
-    cam_super(lanes, sw, sh);
+    int sw = 32, sh = 1;
+    if (lanes > 0) cam_super(lanes, sw, sh);
     a.n_super = (n + sw * sh - 1) / (sw * sh);
   }
   a.rays = rays;
