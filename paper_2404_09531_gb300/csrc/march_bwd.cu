@@ -431,7 +431,9 @@ __device__ __forceinline__ void warp_mlp_input_grad(float* __restrict__ rows, co
 // its own texels (85 % busy, 19 x 16-byte reductions per sample, each lane a
 // wavefront of its own); with 64-byte rows it is 48 % busy and the chain of
 // one queue's steps bounds it.  2^18 rays (field) 866 -> 839 us, 2^20 rays
-// (city) FP32 7.33 -> 6.89, BF16 6.52 -> 6.27 ms per step.  (Staging the rows
+// (city) FP32 7.33 -> 6.89, BF16 6.52 -> 6.27 ms per step (and 6.58 -> 6.57,
+// 5.93 -> 5.75 ms with two channels per FMA and predicated reductions); half of the march's
+// instructions are still the scatter's.  (Staging the rows
 // in shared memory instead of shuffling took 0.97 and 7.95 ms.)
 struct QuadDt {
   float v[4][4];  // [sample of the quad][channel of this lane's half]
@@ -455,10 +457,25 @@ __device__ __forceinline__ unsigned run_ends(int key, bool act, int lane) {
   return __ballot_sync(kFull, act && ((lane & 3) == 3 || next != key));
 }
 
-__device__ __forceinline__ void red4(float* p, const float v[4]) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(v[0]),
-               "f"(v[1]), "f"(v[2]), "f"(v[3])
-               : "memory");
+// Add 4 channels at p where `on`, predicated rather than branched around.
+__device__ __forceinline__ void red4(float* p, float2 lo, float2 hi, bool on) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n @q red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"l"(
+          __cvta_generic_to_global(p)),
+      "f"(lo.x), "f"(lo.y), "f"(hi.x), "f"(hi.y), "r"((unsigned)on)
+      : "memory");
+}
+
+// acc = w v, added to the run's sum unless a run starts here (a sum that is
+// not finite must not reach the next run, so it is selected away, not
+// multiplied by zero).
+__device__ __forceinline__ void run_add(float2 acc[2], float w, const float v[4], bool first) {
+  const float2 ww = make_float2(w, w);
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    if (first) acc[h] = make_float2(0.0f, 0.0f);
+    acc[h] = __ffma2_rn(ww, make_float2(v[2 * h], v[2 * h + 1]), acc[h]);
+  }
 }
 
 // The 4 rows (dx, dy) of the grid cell; off[8] and f[3] are this lane's sample's.
@@ -466,43 +483,44 @@ __device__ __forceinline__ void scatter_grid(const Geo& g, float* __restrict__ b
                                              const QuadDt& q, bool act, int lane) {
   const unsigned ends = run_ends(act && off[0] >= 0 ? off[0] : -1 - lane, act, lane) >> (lane & 28);
   const bool up = (lane >> 1) & 1;
-  float acc[4][4];
+  float* base = buf + 4 * (lane & 1);
+  float2 acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     const float fx = __shfl_sync(kFull, f[0], i, 4), fy = __shfl_sync(kFull, f[1], i, 4),
                 fz = __shfl_sync(kFull, f[2], i, 4);
     const float wz = up ? fz : 1.0f - fz;
-    const bool first = i == 0 || ((ends >> (i - 1)) & 1u), last = (ends >> i) & 1u;
+    const bool last = (ends >> i) & 1u;
+    const bool first = i == 0 || ((ends >> (i - 1)) & 1u);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
       const int lo = __shfl_sync(kFull, off[2 * r], i, 4), hi = __shfl_sync(kFull, off[2 * r + 1], i, 4);
       const float w = ((r & 2) ? fx : 1.0f - fx) * ((r & 1) ? fy : 1.0f - fy) * wz;
-#pragma unroll
-      for (int c = 0; c < 4; c++) acc[r][c] = fmaf(w, q.v[i][c], first ? 0.0f : acc[r][c]);
+      run_add(acc[r], w, q.v[i], first);
       const int o = up ? hi : lo;
-      if (last && o >= 0 && in_range(g, 0, o)) red4(buf + o + 4 * (lane & 1), acc[r]);
+      red4(base + o, acc[r][0], acc[r][1], last && o >= 0 && in_range(g, 0, o));
     }
   }
 }
 
-// The 2 rows of a plane footprint: base texel `base`, row stride `su` elements.
-__device__ __forceinline__ void scatter_plane(const Geo& g, int array, float* __restrict__ buf, int base, int su,
+// The 2 rows of a plane footprint: base texel `at`, row stride `su` elements.
+__device__ __forceinline__ void scatter_plane(const Geo& g, int array, float* __restrict__ buf, int at, int su,
                                               float fu, float fv, const QuadDt& q, bool act, int lane) {
-  const unsigned ends = run_ends(act ? base : -1 - lane, act, lane) >> (lane & 28);
+  const unsigned ends = run_ends(act ? at : -1 - lane, act, lane) >> (lane & 28);
   const bool up = (lane >> 1) & 1;
-  float acc[2][4];
+  float* base = buf + 4 * (lane & 1) + (up ? kNch : 0);
+  float2 acc[2][2];
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     const float u = __shfl_sync(kFull, fu, i, 4), v = __shfl_sync(kFull, fv, i, 4);
-    const int o = __shfl_sync(kFull, base, i, 4) + (up ? kNch : 0);
+    const int o = __shfl_sync(kFull, at, i, 4);
     const float wv = up ? v : 1.0f - v;
-    const bool first = i == 0 || ((ends >> (i - 1)) & 1u), last = (ends >> i) & 1u;
+    const bool last = (ends >> i) & 1u;
+    const bool first = i == 0 || ((ends >> (i - 1)) & 1u);
 #pragma unroll
     for (int r = 0; r < 2; r++) {
-      const float w = (r ? u : 1.0f - u) * wv;
-#pragma unroll
-      for (int c = 0; c < 4; c++) acc[r][c] = fmaf(w, q.v[i][c], first ? 0.0f : acc[r][c]);
-      if (last && in_range(g, array, o + r * su)) red4(buf + o + r * su + 4 * (lane & 1), acc[r]);
+      run_add(acc[r], (r ? u : 1.0f - u) * wv, q.v[i], first);
+      red4(base + o + r * su, acc[r][0], acc[r][1], last && in_range(g, array, o + r * su + (up ? kNch : 0)));
     }
   }
 }
@@ -1191,9 +1209,9 @@ __global__ void __launch_bounds__(128, 1) mlp_bwd_tc_kernel(const Geo g, const B
 // Kernel 2: re-march every ray (one warp per bundle of 32 rays, persistent)
 // and scatter the per-sample gradients.
 // CTAs of 4 warps, 5 per SM (96 registers): the warps take bundles on their
-// own, so small CTAs only set the register granularity.  City step (2^20 rays,
-// FP32 / BF16 features) with 4, 5, 6 CTAs per SM: 7.12 / 6.44, 6.89 / 6.27,
-// 7.52 / 6.84 ms (6 spills).
+// own, so small CTAs only set the register granularity.  City step of 2^20
+// rays (BF16 / FP32) with 5 CTAs per SM 5.75 / 6.57 ms, with 4 5.87 / 6.65
+// ms; 6 spill.
 constexpr int kMarchThreads = 128;
 
 template <class FT, bool SPARSE>
