@@ -18,6 +18,9 @@ OMERF_BF16 = 1
 MLP_NPARAM = 883
 
 
+_PARAM_KEYS = ("grid", "p_xy", "p_xz", "p_yz", "occ", "mlp")
+
+
 class OmerfError(RuntimeError):
     """A negative status returned by the library, with its message."""
 
@@ -449,10 +452,10 @@ def train_fwd(scene, rays, target, smooth_dirs=None, lam=(1.0, 1e-2, 0.0), strea
 def zero_grads(scene):
     """Zeroed float32 gradient buffers shaped like the scene's parameters
     (keys grid, p_xy, p_xz, p_yz, occ, mlp), as the training calls take them."""
-    z = lambda t: torch.zeros(t.shape, dtype=torch.float32, device=t.device)  # noqa: E731
-    return {"grid": z(scene.grid), "p_xy": z(scene.p_xy), "p_xz": z(scene.p_xz), "p_yz": z(scene.p_yz),
-            "occ": z(scene.occ), "mlp": z(scene.mlp)}
-
+    grads = {k: torch.empty(getattr(scene, k).shape, dtype=torch.float32, device=getattr(scene, k).device)
+             for k in _PARAM_KEYS}
+    torch._foreach_zero_(list(grads.values()))  # one launch for all six
+    return grads
 
 
 def train_bwd(scene, saved, inputs, lam=(1.0, 1e-2, 0.0), grad_scale=None, grads=None, stream=None):
@@ -762,7 +765,7 @@ class Trainer:
         self.step_no = 0
         self.grads = zero_grads(scene)
         self.master, self.shadow = {}, {}
-        for k in ("grid", "p_xy", "p_xz", "p_yz", "occ", "mlp"):
+        for k in _PARAM_KEYS:
             t = getattr(scene, k)
             if t.dtype == torch.float32:
                 self.master[k], self.shadow[k] = t, None
@@ -777,8 +780,7 @@ class Trainer:
         gradients before the Adam step."""
         lam7 = lambda_occ(self.step_no) if self.lam_occ is None else self.lam_occ
         lam = (self.lam_rgb, self.lam_smooth, lam7)
-        for g in self.grads.values():
-            g.zero_()
+        torch._foreach_zero_(list(self.grads.values()))
         n = int(torch.as_tensor(rays).shape[0])
         if self.saved is None or self.saved.numel() < n * saved_bytes_per_ray() // 4:
             self.saved = torch.empty(max(n, 1) * saved_bytes_per_ray() // 4, dtype=torch.float32,
