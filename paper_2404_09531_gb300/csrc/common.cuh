@@ -158,26 +158,19 @@ __device__ __forceinline__ bool lattice_test(const Geo& g, const float o[3], con
   return zb.x < p[2] && p[2] < zb.y;
 }
 
-// lattice_test for a caller that keeps the last cell it read and that cell's
-// interval: neighbouring samples of a ray mostly fall into one cell.
-__device__ __forceinline__ bool lattice_test_cached(const Geo& g, const float o[3], const float d[3], int k,
-                                                    float p[3], float2& zb, int& cell) {
-  float t = __fmul_rn((float)k, g.step);
+// The parts of lattice_test: the position of lattice index k, and the cell
+// of a position inside the closed box (float32, no fused operations).
+__device__ __forceinline__ void lattice_point(const Geo& g, const float o[3], const float d[3], int k, float p[3]) {
+  const float t = __fmul_rn((float)k, g.step);
 #pragma unroll
   for (int a = 0; a < 3; a++) p[a] = __fadd_rn(o[a], __fmul_rn(t, d[a]));
-  if (!(p[0] >= g.lo[0] && p[0] <= g.hi[0] && p[1] >= g.lo[1] && p[1] <= g.hi[1] && p[2] >= g.lo[2] &&
-        p[2] <= g.hi[2]))
-    return false;
+}
+__device__ __forceinline__ int occ_cell(const Geo& g, const float p[3]) {
   int cx = (int)floorf(__fmul_rn(__fsub_rn(p[0], g.lo[0]), g.osx));
   int cy = (int)floorf(__fmul_rn(__fsub_rn(p[1], g.lo[1]), g.osy));
   cx = min(max(cx, 0), g.M - 1);
   cy = min(max(cy, 0), g.M - 1);
-  const int c = cx * g.M + cy;
-  if (c != cell) {
-    cell = c;
-    zb = __ldg(g.occ + c);
-  }
-  return zb.x < p[2] && p[2] < zb.y;
+  return cx * g.M + cy;
 }
 
 // Empty-space skipping (Sec. 4.4: max-pooled occupancy planes and box tests).

@@ -12,26 +12,29 @@
 //   G = 1  one lane per ray; the four lanes of a 2 x 2 pixel quad share a
 //          lattice frame, so the lanes of a load group sample one depth (254
 //          wavefronts per 32 samples by a replay, 293 without the frame)
-//   G = 4, 8  the lanes of a ray take consecutive lattice indices: a ray's
+//   G = 4, 8  the lanes of a ray take its next samples together: a ray's
 //          serial chain is 4 or 8 times shorter and there are 4 or 8 times
 //          the warps, for images too small to fill the chip with G = 1
 // A frame skips the 32-index windows that the coarse occupancy grid rules
-// out.  Texel pairs are read in even / odd order (216 wavefronts, see
-// even_odd) with two channels per FMA.  All forms composite a ray's samples
-// one after the other in the same order, so a pixel does not depend on G, nor
-// on whether counts are wanted.
+// out, tests a whole window at a time and then takes the evaluated samples.
+// Texel pairs are read in even / odd order (216 wavefronts, see even_odd)
+// with two channels per FMA.  All forms composite a ray's samples one after
+// the other in the same order, so a pixel does not depend on G, nor on
+// whether counts are wanted.
 //
 // Measured on a GB300, 512 x 512 x 32 city, against the packed queue:
-// 8 x 1920x1080 29.4 -> 21.0 ms (L1 pipe 86 % busy), 1920x1080 3.80 -> 2.73
-// ms (G = 4: 3.11), 641x361 0.84 -> 0.45 ms (G = 8: 0.50, G = 1: 0.91),
-// 64x64 of the 64 x 64 x 16 field 0.155 -> 0.058 ms (G = 4: 0.080).
+// 8 x 1920x1080 29.4 -> 20.3 ms (L1 pipe 83 % busy, 1.8 G instead of 2.7 G
+// instructions per frame), 1920x1080 3.80 -> 2.55 ms (G = 4: 3.01), 640x360
+// 0.83 -> 0.46 ms (G = 8: 0.49, G = 1: 0.83), 64x64 of the 64 x 64 x 16 field
+// 0.155 -> 0.053 ms (G = 4: 0.064).
 //
-// Sample counts are those of the packed queue, which training and ray lists
-// use, also where rounding decides them.  The two forms multiply a ray's
-// transmittance in different orders: where counts are wanted the density is
-// also summed in the queue's order, its transmittance decides the count, and
-// a ray that passes the termination threshold within the products' rounding
-// (about 1 of 10^5) is counted again by marching its tile with the queue.
+// Sample counts are those of the packed queue, which training and long ray
+// lists use, also where rounding decides them.  The two forms multiply a
+// ray's transmittance in different orders: where counts are wanted the
+// density is also summed in the queue's order, its transmittance decides the
+// count, and a ray that passes the termination threshold within the
+// products' rounding (about 1 of 10^5) is counted again by marching its
+// bundle with the queue.
 #include "march_fwd.cuh"
 
 namespace omerf {
@@ -72,62 +75,123 @@ __device__ __forceinline__ void lane_pixel(int warp, int lane, int& x, int& y) {
   }
 }
 
-// mlp_forward_padded with the units of each layer spread over the G lanes of
-// a ray (every unit summed in the same order): output j is lane j's return
-// value, j < 3.  All lanes of the warp call it.
-template <int G>
-__device__ __forceinline__ float mlp_group(const float* __restrict__ W, const float F[7], const float d[3], int j) {
-  float sc[(12 + G - 1) / G][2];
-#pragma unroll
-  for (int i = 0; i < (12 + G - 1) / G; i++) {
-    const int m = min(i * G + j, 11), k = m / 3, a = m - 3 * k;
-    const float da = a == 0 ? d[0] : (a == 1 ? d[1] : d[2]);
-    sincosf((float)(1 << k) * da, &sc[i][0], &sc[i][1]);
+// The deferred MLP's weights with the units of a layer as the fast axis, so that
+// two units share one packed FMA: W1 [34][16], b1 [16], W2 [16][16], b2 [16],
+// W3 [16][4 (3 used)], b3 [4 (3 used)].
+constexpr int kTW1 = 0, kTB1 = 544, kTW2 = 560, kTB2 = 816, kTW3 = 832, kTB3 = 896, kSmemMlpT = 900;
+
+__device__ __forceinline__ void load_mlp_units(const float* __restrict__ gw, float* __restrict__ sw) {
+  for (int i = threadIdx.x; i < kSmemMlpT; i += blockDim.x) {
+    float v = 0.0f;
+    if (i < kTB1) v = gw[kOffW1 + (i & 15) * 34 + (i >> 4)];
+    else if (i < kTW2) v = gw[kOffB1 + i - kTB1];
+    else if (i < kTB2) v = gw[kOffW2 + ((i - kTW2) & 15) * 16 + ((i - kTW2) >> 4)];
+    else if (i < kTW3) v = gw[kOffB2 + i - kTB2];
+    else if (i < kTB3) v = ((i - kTW3) & 3) < 3 ? gw[kOffW3 + ((i - kTW3) & 3) * 16 + ((i - kTW3) >> 2)] : 0.0f;
+    else v = i - kTB3 < 3 ? gw[kOffB3 + i - kTB3] : 0.0f;
+    sw[i] = v;
   }
-  float x[36];
+}
+
+// N units from u0 of one layer: h = relu(b + sum_i x_i W[i][u]), two units per FMA.
+template <int N, int IN>
+__device__ __forceinline__ void mlp_units(const float* __restrict__ W, const float* __restrict__ b, int u0,
+                                          const float x[IN], float h[N]) {
+  float2 acc[N / 2];
+#pragma unroll
+  for (int q = 0; q < N / 2; q++) acc[q] = *reinterpret_cast<const float2*>(b + u0 + 2 * q);
+#pragma unroll
+  for (int i = 0; i < IN; i++) {
+    const float2 xx = make_float2(x[i], x[i]);
+#pragma unroll
+    for (int q = 0; q < N / 4; q++) {
+      const float4 w = *reinterpret_cast<const float4*>(W + 16 * i + u0 + 4 * q);
+      acc[2 * q] = __ffma2_rn(xx, make_float2(w.x, w.y), acc[2 * q]);
+      acc[2 * q + 1] = __ffma2_rn(xx, make_float2(w.z, w.w), acc[2 * q + 1]);
+    }
+    if (N == 2) acc[0] = __ffma2_rn(xx, *reinterpret_cast<const float2*>(W + 16 * i + u0), acc[0]);
+  }
+#pragma unroll
+  for (int q = 0; q < N / 2; q++) {
+    h[2 * q] = fmaxf(acc[q].x, 0.0f);
+    h[2 * q + 1] = fmaxf(acc[q].y, 0.0f);
+  }
+}
+
+// G(F, d) with the units of each layer spread over the G lanes of a ray (every
+// unit summed in the same order whatever G): all three outputs for G = 1,
+// output j in y[0] of lane j < 3 else.  sin and cos of 2, 4 and 8 d follow from
+// those of d by doubling (each doubling at most doubles the error: below 1e-6).
+// All lanes of the warp call it for G > 1.  The render of a 1080p frame spent
+// 0.39 of 2.83 ms here with twelve sincosf and one unit per FMA.
+template <int G>
+__device__ __forceinline__ void mlp_rays(const float* __restrict__ W, const float F[7], const float d[3], int j,
+                                         float y[3]) {
+  constexpr int N = 16 / G;
+  float x[34], h[N], a[16];
 #pragma unroll
   for (int i = 0; i < 7; i++) x[i] = F[i];
 #pragma unroll
-  for (int a = 0; a < 3; a++) x[7 + a] = d[a];
+  for (int c = 0; c < 3; c++) {
+    float s, co;
+    sincosf(d[c], &s, &co);
+    x[7 + c] = d[c];
 #pragma unroll
-  for (int m = 0; m < 12; m++) {
-    const int k = m / 3, a = m % 3;
-    x[10 + 6 * k + a] = __shfl_sync(kFull, sc[m / G][0], m % G, G);
-    x[10 + 6 * k + 3 + a] = __shfl_sync(kFull, sc[m / G][1], m % G, G);
+    for (int k = 0; k < 4; k++) {
+      x[10 + 6 * k + c] = s;
+      x[13 + 6 * k + c] = co;
+      const float s2 = 2.0f * s;
+      co = fmaf(-s2, s, 1.0f);
+      s = s2 * x[13 + 6 * k + c];
+    }
   }
-  x[34] = 0.0f;
-  x[35] = 0.0f;
-  float h[16 / G];
+  mlp_units<N, 34>(W + kTW1, W + kTB1, N * j, x, h);
 #pragma unroll
-  for (int i = 0; i < 16 / G; i++) {
-    const int u = i * G + j;
-    const float4* w = reinterpret_cast<const float4*>(W + kSW1 + 36 * u);
-    float a = W[kSB1 + u];
+  for (int u = 0; u < 16; u++) a[u] = G == 1 ? h[u % N] : __shfl_sync(kFull, h[u % N], u / N, G);
+  mlp_units<N, 16>(W + kTW2, W + kTB2, N * j, a, h);
 #pragma unroll
-    for (int q = 0; q < 9; q++) a = dot4(w[q], x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3], a);
-    h[i] = fmaxf(a, 0.0f);
+  for (int u = 0; u < 16; u++) a[u] = G == 1 ? h[u % N] : __shfl_sync(kFull, h[u % N], u / N, G);
+  if (G == 1) {
+    float2 o[2] = {make_float2(W[kTB3], W[kTB3 + 1]), make_float2(W[kTB3 + 2], 0.0f)};
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const float4 w = *reinterpret_cast<const float4*>(W + kTW3 + 4 * i);
+      const float2 xx = make_float2(a[i], a[i]);
+      o[0] = __ffma2_rn(xx, make_float2(w.x, w.y), o[0]);
+      o[1] = __ffma2_rn(xx, make_float2(w.z, w.w), o[1]);
+    }
+    y[0] = sigmoidf_(o[0].x);
+    y[1] = sigmoidf_(o[0].y);
+    y[2] = sigmoidf_(o[1].x);
+  } else {
+    const int o = min(j, 2);
+    float v = W[kTB3 + o];
+#pragma unroll
+    for (int i = 0; i < 16; i++) v = fmaf(a[i], W[kTW3 + 4 * i + o], v);
+    y[0] = sigmoidf_(v);
   }
-  float h1[16];
-#pragma unroll
-  for (int u = 0; u < 16; u++) h1[u] = __shfl_sync(kFull, h[u / G], u % G, G);
-#pragma unroll
-  for (int i = 0; i < 16 / G; i++) {
-    const int u = i * G + j;
-    const float4* w = reinterpret_cast<const float4*>(W + kSW2 + 16 * u);
-    float a = W[kSB2 + u];
-#pragma unroll
-    for (int q = 0; q < 4; q++) a = dot4(w[q], h1[4 * q], h1[4 * q + 1], h1[4 * q + 2], h1[4 * q + 3], a);
-    h[i] = fmaxf(a, 0.0f);
+}
+
+// The evaluated lattice indices of a window, [k0, k0 + 31] clipped to the ray's
+// [klo, khi]: every lane of a ray tests 32 / G of them with the decision rule.
+// A run of tests without votes or branches in between: one candidate per
+// step of the march, with a vote each, took 36 % of a frame's instructions.
+template <int G>
+__device__ __forceinline__ unsigned window_samples(const Geo& g, const float o[3], const float d[3], int k0, int klo,
+                                                   int khi, int j) {
+  unsigned m = 0;
+#pragma unroll 8
+  for (int i = 0; i < 32; i += G) {
+    float p[3];
+    lattice_point(g, o, d, k0 + i + j, p);
+    const bool in = p[0] >= g.lo[0] && p[0] <= g.hi[0] && p[1] >= g.lo[1] && p[1] <= g.hi[1] && p[2] >= g.lo[2] &&
+                    p[2] <= g.hi[2];
+    float2 zb = make_float2(0.0f, 0.0f);
+    if (in) zb = __ldg(g.occ + occ_cell(g, p));
+    if (in && zb.x < p[2] && p[2] < zb.y) m |= 1u << (i + j);
   }
-  float h2[16];
-#pragma unroll
-  for (int u = 0; u < 16; u++) h2[u] = __shfl_sync(kFull, h[u / G], u % G, G);
-  const int o = min(j, 2);
-  const float4* w = reinterpret_cast<const float4*>(W + kSW3 + 16 * o);
-  float a = W[kSB3 + o];
-#pragma unroll
-  for (int q = 0; q < 4; q++) a = dot4(w[q], h2[4 * q], h2[4 * q + 1], h2[4 * q + 2], h2[4 * q + 3], a);
-  return sigmoidf_(a);
+  const int lo = max(klo - k0, 0), hi = min(khi - k0, 31);
+  return lo > hi ? 0u : m & (~0u << lo) & (~0u >> (31 - hi));
 }
 
 // The bits of a ballot that belong to the lanes of this lane's ray.
@@ -210,18 +274,19 @@ __device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, Warp
   if (valid && ((want >> lane) & 1u)) a.count[rid] = ws.s.cnt[lane];
 }
 
-// 7 CTAs of 4 warps (72 registers) per SM: 2.91 ms per 1080p frame, 2.90 with
-// 6, 3.07 with 8, 2.94 with 5.
+// Resident CTAs per SM (1080p frame with 6, 7, 8 for G = 1: 2.55, 2.58, 2.58
+// ms; 640x360 with 6, 7 for G = 4: 455, 476 us; 320x180 with 6, 7 for G = 8:
+// 242, 208 us); the counting form keeps its second density sum in registers.
 template <class FT, bool SPARSE, int G, bool COUNT>
-__global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
+__global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 ? 7 : 6))
     march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
   constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
   constexpr unsigned kFrameMask = (1u << kFrame) - 1u;
   constexpr int kTilesX = (CamShape<G>::kW + 7) / 8, kTilesY = (CamShape<G>::kH + 3) / 4;
-  __shared__ __align__(16) float sW[kSmemMlp];
+  __shared__ __align__(16) float sW[kSmemMlpT];
   __shared__ typename std::conditional<COUNT, WarpMarch<false>, int>::type sMarch;
   __shared__ unsigned sWork[2], sAmb[kTilesX * kTilesY];
-  load_mlp_padded(g.mlp, sW);
+  load_mlp_units(g.mlp, sW);
   if (COUNT && threadIdx.x < kTilesX * kTilesY) sAmb[threadIdx.x] = 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int base = lane & ~(kFrame - 1), j = G == 1 ? 0 : lane & (G - 1);
@@ -262,31 +327,30 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
       klo = 0x7fffffff;
       khi = -1;
     }
-    // the common lattice frame
-    int k = klo, ke = khi;
+    // the common lattice frame and its blocks of 32 windows from wb
+    int wb = klo, ke = khi;
     if (G == 1) {
-      k = min(k, __shfl_xor_sync(kFull, k, 1));
-      k = min(k, __shfl_xor_sync(kFull, k, 2));
+      wb = min(wb, __shfl_xor_sync(kFull, wb, 1));
+      wb = min(wb, __shfl_xor_sync(kFull, wb, 2));
       ke = max(ke, __shfl_xor_sync(kFull, ke, 1));
       ke = max(ke, __shfl_xor_sync(kFull, ke, 2));
     }
-    int wb = k;
     unsigned wm = 0;
-    bool need_mask = true, amb = false, done = false, counted = false;
+    bool need_mask = wb <= ke;
+    bool amb = false, done = false, counted = false;
     float T = 1.0f, Tc = 1.0f, F[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    int seen = 0, cnt = 0, ccell = -1;
-    float2 zb = make_float2(0.0f, 0.0f);
-    while (__any_sync(kFull, k <= ke)) {
-      // advance every frame to its next lattice index (or G of them) at which
-      // a ray is evaluated
-      bool hit = false, need = k <= ke;
-      unsigned hits = 0;
-      float p[3] = {0.0f, 0.0f, 0.0f};
-      while (__any_sync(kFull, need)) {
-        if (__any_sync(kFull, need_mask)) {
-          // windows of 32 indices that the coarse grid cannot rule out
+    int seen = 0, cnt = 0;
+    int k0 = 0;
+    unsigned own = 0, todo = 0;
+    for (;;) {
+      // A frame whose window is done takes its next one that the coarse grid
+      // cannot rule out.  With one lane per ray the frames of a warp do so
+      // together (a window is 32 tests for every lane), else each when it has to.
+      if (G > 1 || !__any_sync(kFull, todo != 0u)) {
+        while (__any_sync(kFull, todo == 0u && need_mask)) {
+          const bool now = todo == 0u && need_mask;
           unsigned m = 0;
-          if (need_mask && alive) {
+          if (now && alive) {
             const int nw = min((ke - wb) >> 5, 31);
             for (int jw = j; jw <= nw; jw += G) {
               const int ka = max(wb + 32 * jw, klo), kz = min(wb + 32 * jw + 31, khi);
@@ -295,34 +359,52 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
           }
 #pragma unroll
           for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
-          if (need_mask) wm = m;
-          need_mask = false;
-        }
-        bool h = false;
-        if (need) {
-          const int off = k - wb;
-          if (off >= 1024) {
-            wb = k;
-            need_mask = true;
-          } else {
-            const unsigned rem = wm & (~0u << (off >> 5));
-            const int jn = __ffs(rem) - 1;
-            if (rem == 0) {
-              k = wb + 1024;
-            } else {
-              if (jn > (off >> 5)) k = wb + 32 * jn;
-              const int kk = k + j;
-              h = alive && kk >= klo && kk <= khi && lattice_test_cached(g, o, d, kk, p, zb, ccell);
-              k += G;
-            }
+          if (now) {
+            wm = m;
+            need_mask = wm == 0u && wb + 1024 <= ke;
+            if (need_mask) wb += 1024;
           }
         }
-        const unsigned hb = __ballot_sync(kFull, h);
-        if (need) {
-          hit = h;
-          hits = (hb >> base) & kFrameMask;
-          need = hits == 0u && k <= ke;
+        if (__any_sync(kFull, todo == 0u && wm != 0u)) {
+          // the window's evaluated indices (bit i: index k0 + i): of this
+          // lane's ray (own), and of any ray of the frame (todo)
+          const bool now = todo == 0u && wm != 0u;
+          unsigned m = 0;
+          if (now) {
+            k0 = wb + 32 * (__ffs(wm) - 1);
+            if (alive) m = window_samples<G>(g, o, d, k0, klo, khi, j);
+            own = m;
+            wm &= wm - 1u;
+            need_mask = wm == 0u && wb + 1024 <= ke;
+            if (need_mask) wb += 1024;
+          }
+#pragma unroll
+          for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
+          if (now) todo = m;
+          continue;
         }
+        if (!__any_sync(kFull, todo != 0u)) break;
+      }
+      // G = 1: the frame's next index, for the rays evaluated there; else the
+      // ray's next G samples, one per lane
+      unsigned left = todo;
+      if (G == 1) {
+        todo &= todo - 1u;
+      } else {
+#pragma unroll
+        for (int i = 0; i < G - 1; i++) {
+          if (i < j) left &= left - 1u;
+          todo &= todo - 1u;
+        }
+        todo &= todo - 1u;
+      }
+      const int bit = __ffs(left) - 1;
+      bool hit = alive && left != 0u && (G != 1 || ((own >> bit) & 1u));
+      float p[3] = {0.0f, 0.0f, 0.0f};
+      float2 zb = make_float2(0.0f, 0.0f);
+      if (hit) {
+        lattice_point(g, o, d, k0 + bit, p);
+        zb = __ldg(g.occ + occ_cell(g, p));
       }
       if (G == 1) {
         if (hit) {
@@ -349,10 +431,12 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
           alive = seen < g.n_max && !(done && (!COUNT || counted));
         }
         const unsigned am = __ballot_sync(kFull, alive);
-        if (((am >> base) & kFrameMask) == 0u) k = ke + 1;
+        if (((am >> base) & kFrameMask) == 0u) {
+          todo = wm = 0u;
+          need_mask = false;
+        }
       } else {
-        const int rank = __popc(hits & ((1u << j) - 1u));  // this frame's samples before this lane's
-        hit = hit && seen + rank < g.n_max;
+        hit = hit && seen + j < g.n_max;
         SampleAct s;
         s.ah = 0.0f;
         float ahc = 0.0f;
@@ -401,8 +485,8 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
         }
         seen += __popc(hits_of<G>(hit, base));
         if (seen >= g.n_max || (done && (!COUNT || counted))) {
-          alive = false;
-          k = ke + 1;
+          alive = need_mask = false;
+          todo = wm = 0u;
         }
       }
     }
@@ -411,7 +495,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
     if (G == 1) {
       if (valid) {
         float yd[3] = {0.0f, 0.0f, 0.0f};
-        if (seen > 0) mlp_forward_padded(sW, F, d, yd);
+        if (seen > 0) mlp_rays<1>(sW, F, d, 0, yd);
 #pragma unroll
         for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T, g.bg[c], F[c] + yd[c]) : g.bg[c];
 #pragma unroll
@@ -419,11 +503,11 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : 7)
         if (COUNT) a.count[rid] = cnt;
       }
     } else {
-      float y = 0.0f;
-      if (__any_sync(kFull, seen > 0)) y = mlp_group<G>(sW, F, d, j);
+      float y[3] = {0.0f, 0.0f, 0.0f};
+      if (__any_sync(kFull, seen > 0)) mlp_rays<G>(sW, F, d, j, y);
       if (valid && j < 3) {
         const float Fj = j == 0 ? F[0] : (j == 1 ? F[1] : F[2]);
-        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T, g.bg[j], Fj + y) : g.bg[j];
+        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T, g.bg[j], Fj + y[0]) : g.bg[j];
         if (COUNT && j == 0) a.count[rid] = cnt;
       }
     }
@@ -473,14 +557,14 @@ static cudaError_t launch_cam_group(const omerf_scene* s, const FwdArgs& a, cuda
 }
 
 // The lines lie where the measured times cross (us with 8 / 4 / 1 lanes; city
-// unless said): 57,600 rays 212 / 286 / 781, 129,600 rays 343 / 350 / 865,
-// 230,400 rays 542 / 478 / 998, 921,600 rays 1935 / 1520 / 1593, 1,048,576
-// rays (field) 996 / 721 / 604, 1,398,784 rays 3183 / 2450 / 2212.  A BF16
+// unless said): 57,600 rays 208 / 267 / 549, 129,600 rays 320 / 331 / 711,
+// 230,400 rays 490 / 455 / 833, 518,400 rays 1003 / 852 / 1027, 921,600 rays
+// 1708 / 1419 / 1387, 1,048,576 rays (field) 848 / 632 / 469.  A BF16
 // scene keeps the packed queue: its deferred MLP rounds F to bfloat16, so sums
 // in another order would move pixels by a step of that rounding.
 int cam_lanes(const omerf_scene* s, long n) {
   if (s->desc.feat_dtype != OMERF_F32) return 0;
-  return n < (1 << 17) ? 8 : (n < (1 << 20) ? 4 : 1);
+  return n < (1 << 17) ? 8 : (n < (3 << 18) ? 4 : 1);
 }
 
 // Rays of a list may lie anywhere: rays of different lengths share a warp, and
