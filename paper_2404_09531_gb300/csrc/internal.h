@@ -108,6 +108,6 @@ omerf_status output_ptr(void* p, void** dev, const char* name);
 omerf::Cam to_cam(const omerf_camera* c);
 
 namespace omerf {
-__global__ void hull_kernel(const float2* __restrict__ occ, long cells, float* __restrict__ hull);
-__global__ void coarse_hull_kernel(const float2* __restrict__ occ, int M, int clog2, int Mc, float2* __restrict__ chull);
+// Rebuild a scene's coarse occupancy grid and hull from its occupancy plane.
+cudaError_t launch_hulls(const omerf_scene* s, cudaStream_t stream);
 }  // namespace omerf

@@ -127,12 +127,8 @@ extern "C" omerf_status omerf_render_noalloc(const omerf_scene_desc* desc, const
   // whatever the previous call (of any scene) left in it.  The work counter
   // is zeroed by the launch.
   cudaStream_t cs = (cudaStream_t)stream;
-  const long occ_cells = (long)desc->occ_res * desc->occ_res;
   OMERF_LAUNCH_FAULT();
-  hull_kernel<<<1, 1024, 0, cs>>>(s.geo.occ, occ_cells, s.state);
-  coarse_hull_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, cs>>>(s.geo.occ, desc->occ_res, s.clog2, s.Mc,
-                                                                      s.chull);
-  e = cudaGetLastError();
+  e = launch_hulls(&s, cs);
   if (e != cudaSuccess) return cuda_fail(e, "no-allocation hull kernels");
   if (nbr_bytes && (st = build_brick_neighbors(&s, cs)) != OMERF_OK) return st;
   e = launch_march_fwd(&s, cam ? &k : nullptr, rays, n, rgb, count, nullptr, nullptr, 0, nullptr, nullptr, nullptr,

@@ -36,8 +36,8 @@ unsigned* next_counter(const omerf_scene* s, cudaStream_t stream) {
 // ---------------------------------------------------------------------------
 // One block (no second pass, no atomics): the loads of eight rounds are in
 // flight together (65,536 cells 10.0 us, 13.0 us one round at a time).
-__global__ void __launch_bounds__(1024) hull_kernel(const float2* __restrict__ occ, long cells,
-                                                    float* __restrict__ hull) {
+static __global__ void __launch_bounds__(1024) hull_kernel(const float2* __restrict__ occ, long cells,
+                                                           float* __restrict__ hull) {
   __shared__ float slo[32], shi[32];
   float lo = __int_as_float(0x7f800000), hi = -lo;
   for (long i0 = threadIdx.x; i0 < cells; i0 += 8 * blockDim.x) {
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(1024) hull_kernel(const float2* __restrict__ o
 // Coarse max-pooled occupancy grid (Sec. 4.4: 2D max pooling of the occupancy
 // plane for empty-space skipping): cell (X, Y) holds the min z_min and max
 // z_max over the non-empty occupancy cells it covers, (+inf, -inf) if none.
-__global__ void coarse_hull_kernel(const float2* __restrict__ occ, int M, int clog2, int Mc,
+static __global__ void coarse_hull_kernel(const float2* __restrict__ occ, int M, int clog2, int Mc,
                                    float2* __restrict__ chull) {
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= Mc * Mc) return;
@@ -92,6 +92,16 @@ __global__ void coarse_hull_kernel(const float2* __restrict__ occ, int M, int cl
       }
     }
   chull[id] = make_float2(lo, hi);
+}
+
+// The coarse grid, then the hull over its cells: the same minimum and maximum
+// as over the occupancy plane's, from 4^clog2 times fewer (256^2 plane: 10.0 +
+// 3.9 us with the hull of the whole plane).
+cudaError_t launch_hulls(const omerf_scene* s, cudaStream_t stream) {
+  const int nc = s->Mc * s->Mc;
+  coarse_hull_kernel<<<(nc + 255) / 256, 256, 0, stream>>>(s->geo.occ, s->desc.occ_res, s->clog2, s->Mc, s->chull);
+  hull_kernel<<<1, 1024, 0, stream>>>(s->chull, nc, s->state);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -609,13 +619,8 @@ int64_t omerf_scene_device_bytes(const omerf_scene_desc* desc) {
 omerf_status omerf_scene_update(omerf_scene* s, void* stream) {
   OMERF_API_RANGE();
   if (!s) { set_error("scene is NULL"); return OMERF_EINVAL; }
-  const long cells = (long)s->desc.occ_res * s->desc.occ_res;
   OMERF_LAUNCH_FAULT();
-  hull_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(s->geo.occ, cells, s->state);
-  const int nc = s->Mc * s->Mc;
-  coarse_hull_kernel<<<(nc + 255) / 256, 256, 0, (cudaStream_t)stream>>>(s->geo.occ, s->desc.occ_res, s->clog2,
-                                                                         s->Mc, s->chull);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_hulls(s, (cudaStream_t)stream);
   return e == cudaSuccess ? OMERF_OK : cuda_fail(e, "hull kernel");
 }
 
