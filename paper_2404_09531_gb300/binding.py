@@ -124,6 +124,10 @@ def _check(status: int, what: str):
 
 def _stream(stream=None):
     if stream is None:
+        if torch.cuda.is_initialized():
+            # the current device's current stream, without building a Stream object
+            # around it (about 5 us of every call)
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
@@ -587,16 +591,17 @@ def extract_bricks(grid_res, brick, table, src, src_table=None, n_bricks=None, s
 def plane_crop_rows(scene, stream=None):
     """Rows (k0, k1) of the scene's XZ/YZ planes any evaluated sample reads and
     the cropped z-range, or None if no cell is occupied (one small readback)."""
-    rows = torch.empty(2, dtype=torch.int32, device=scene.device)
-    zr = torch.empty(2, dtype=torch.float32, device=scene.device)
+    both = torch.empty(4, dtype=torch.int32, device=scene.device)  # read back together
+    rows, zr = both[:2], both[2:]
     pz = scene.plane_z if scene.plane_z is not None else (scene.aabb[4], scene.aabb[5])
     _check(lib().omerf_plane_crop_rows((ctypes.c_float * 2)(*pz), int(scene.plane_res[2]), _ptr(scene.occ),
                                        int(scene.occ_res), _ptr(rows), _ptr(zr), _stream(stream)),
            "omerf_plane_crop_rows")
-    r = rows.cpu().tolist()
+    both = both.cpu()
+    r = both[:2].tolist()
     if r[0] < 0:
         return None
-    return (r[0], r[1]), tuple(float(v) for v in zr.cpu().tolist())
+    return (r[0], r[1]), tuple(both[2:].view(torch.float32).tolist())
 
 
 def crop_planes(scene, stream=None):

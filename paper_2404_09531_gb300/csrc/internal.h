@@ -11,6 +11,7 @@
 struct omerf_scene {
   omerf_scene_desc desc;
   omerf::Geo geo;
+  void* block = nullptr;           // device: the one allocation that holds the parts below
   float* state = nullptr;          // device: [0..1] occupancy hull (min z_min, max z_max)
   unsigned* counters = nullptr;    // device: per-launch work counters
   float2* chull = nullptr;         // device: coarse max-pooled occupancy grid [Mc][Mc]
