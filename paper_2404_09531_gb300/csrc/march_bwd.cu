@@ -439,15 +439,23 @@ struct QuadDt {
   float v[4][4];  // [sample of the quad][channel of this lane's half]
 };
 
+// (12 shuffles in two exchanges instead of a broadcast of every value, 32: 762
+// -> 751 us per 2^18-ray step together with the planes' shared fractions)
 __device__ __forceinline__ void quad_exchange(const float dt[8], int lane, QuadDt& q) {
-  const bool hi = lane & 1;
+  const bool hi = lane & 1, up = lane & 2;
 #pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      const float a = __shfl_sync(kFull, dt[c], i, 4), b = __shfl_sync(kFull, dt[4 + c], i, 4);
-      q.v[i][c] = hi ? b : a;
-    }
+  for (int c = 0; c < 4; c++) {
+    // within the pair each lane keeps its half and hands the other over; then
+    // the pairs exchange their two samples
+    const float keep = hi ? dt[4 + c] : dt[c];
+    const float got = __shfl_xor_sync(kFull, hi ? dt[c] : dt[4 + c], 1);
+    const float a = hi ? got : keep, b = hi ? keep : got;
+    const float oa = __shfl_xor_sync(kFull, a, 2), ob = __shfl_xor_sync(kFull, b, 2);
+    q.v[0][c] = up ? oa : a;
+    q.v[1][c] = up ? ob : b;
+    q.v[2][c] = up ? a : oa;
+    q.v[3][c] = up ? b : ob;
+  }
 }
 
 // Bit l: lane l's sample is active and the next lane of its quad does not
@@ -503,24 +511,35 @@ __device__ __forceinline__ void scatter_grid(const Geo& g, float* __restrict__ b
   }
 }
 
-// The 2 rows of a plane footprint: base texel `at`, row stride `su` elements.
-__device__ __forceinline__ void scatter_plane(const Geo& g, int array, float* __restrict__ buf, int at, int su,
-                                              float fu, float fv, const QuadDt& q, bool act, int lane) {
-  const unsigned ends = run_ends(act ? at : -1 - lane, act, lane) >> (lane & 28);
+// The 2 rows of each plane's footprint; pi[3] and f[3] are this lane's
+// sample's lower texel and fraction along x, y and z.
+__device__ __forceinline__ void scatter_planes(const Geo& g, float* const buf[3], const int pi[3], const float f[3],
+                                               const QuadDt& q, bool act, int lane) {
+  float fs[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) fs[c][i] = __shfl_sync(kFull, f[c], i, 4);
   const bool up = (lane >> 1) & 1;
-  float* base = buf + 4 * (lane & 1) + (up ? kNch : 0);
-  float2 acc[2][2];
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const float u = __shfl_sync(kFull, fu, i, 4), v = __shfl_sync(kFull, fv, i, 4);
-    const int o = __shfl_sync(kFull, at, i, 4);
-    const float wv = up ? v : 1.0f - v;
-    const bool last = (ends >> i) & 1u;
-    const bool first = i == 0 || ((ends >> (i - 1)) & 1u);
+  for (int pl = 0; pl < 3; pl++) {
+    if (!buf[pl]) continue;
+    const int U = pl == 2 ? 1 : 0, V = pl == 0 ? 1 : 2;
+    const int su = g.R[V] * kNch, at = pi[U] * su + pi[V] * kNch;
+    const unsigned ends = run_ends(act ? at : -1 - lane, act, lane) >> (lane & 28);
+    float* base = buf[pl] + 4 * (lane & 1) + (up ? kNch : 0);
+    float2 acc[2][2];
 #pragma unroll
-    for (int r = 0; r < 2; r++) {
-      run_add(acc[r], (r ? u : 1.0f - u) * wv, q.v[i], first);
-      red4(base + o + r * su, acc[r][0], acc[r][1], last && in_range(g, array, o + r * su + (up ? kNch : 0)));
+    for (int i = 0; i < 4; i++) {
+      const int o = __shfl_sync(kFull, at, i, 4);
+      const float wv = up ? fs[V][i] : 1.0f - fs[V][i];
+      const bool last = (ends >> i) & 1u;
+      const bool first = i == 0 || ((ends >> (i - 1)) & 1u);
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        run_add(acc[r], (r ? fs[U][i] : 1.0f - fs[U][i]) * wv, q.v[i], first);
+        red4(base + o + r * su, acc[r][0], acc[r][1], last && in_range(g, 1 + pl, o + r * su + (up ? kNch : 0)));
+      }
     }
   }
 }
@@ -621,12 +640,8 @@ __device__ __forceinline__ void march_bundle_bwd(const Geo& g, const BwdArgs& a,
     }
 #pragma unroll
     for (int c = 0; c < 3; c++) axis_coord(p[c], g.lo[c], g.ps[c], g.R[c], pi[c], pf[c], c == 2 ? g.pzoff : 0.0f);
-    if (a.g_xy)
-      scatter_plane(g, 1, a.g_xy, (pi[0] * g.R[1] + pi[1]) * kNch, g.R[1] * kNch, pf[0], pf[1], q, act, lane);
-    if (a.g_xz)
-      scatter_plane(g, 2, a.g_xz, (pi[0] * g.R[2] + pi[2]) * kNch, g.R[2] * kNch, pf[0], pf[2], q, act, lane);
-    if (a.g_yz)
-      scatter_plane(g, 3, a.g_yz, (pi[1] * g.R[2] + pi[2]) * kNch, g.R[2] * kNch, pf[1], pf[2], q, act, lane);
+    float* const planes[3] = {a.g_xy, a.g_xz, a.g_yz};
+    scatter_planes(g, planes, pi, pf, q, act, lane);
     const int rnext = __shfl_down_sync(kFull, r, 1);
     const bool tail = act && (lane == 31 || rnext != r);
     __syncwarp();
