@@ -35,7 +35,7 @@ import synth  # noqa: E402
 
 BYTES_PER_SAMPLE = {"f32": 640 + 8, "bf16": 320 + 8}  # feature gather + occupancy bounds
 BYTES_PER_RAY_RENDER = 12 + 4                          # rgb + count written
-# Sources the dominant kernel (march_fwd_kernel<float, sparse, render>) is
+# Sources the dominant kernel (march_cam_kernel<float, sparse, 1, pixels>) is
 # compiled from: a recorded DRAM traffic figure is valid only for the sources
 # it was captured with.
 RENDER_SOURCES = ("paper_2404_09531_gb300/csrc/march_cam.cu", "paper_2404_09531_gb300/csrc/march_fwd.cu",
@@ -44,7 +44,7 @@ RENDER_SOURCES = ("paper_2404_09531_gb300/csrc/march_cam.cu", "paper_2404_09531_
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of that kernel
 # over the step's eight 1920x1080 cameras (one ncu capture), with the hash of
 # the sources it was captured from.
-TRAFFIC = {"sources_sha256_16": "03170e84b2575a5d", "bytes": 179789568.0 + 176725248.0}
+TRAFFIC = {"sources_sha256_16": "99c9890c87a0fab5", "bytes": 168892928.0 + 175876608.0}
 
 
 def render_sources_hash():
@@ -802,7 +802,7 @@ def run_native(args):
         "msamples_per_s": ws * samples_per_step / (t_step * 1e-3) / 1e6,
         "roofline": {"bound": "l1", "achieved": achieved, "peak": l1, "unit": "GB/s", "frac": achieved / l1,
                      "traffic": traffic_per_launch(),
-                     "kernel": "march_fwd_kernel<float, sparse, render>",
+                     "kernel": "march_cam_kernel<float, sparse, 1, pixels>",
                      "peak_kind": "measured in this run: L1 load bandwidth of the gather's 256-bit read-only load "
                                   "(omerf_probe_load_bandwidth, 3 x 256-thread CTAs per SM, 16 KB slice each)",
                      "algorithmic_bytes_per_launch": bytes_launch,
