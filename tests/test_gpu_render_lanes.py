@@ -59,3 +59,37 @@ def test_short_ray_lists_match_long_ones(cfg, n):
     r = rays[:n].cpu().numpy()[idx]
     ref = oracle.render(oracle_scene_for(sc, table, pool), r)
     compare_render(rgb.cpu().numpy()[idx], cnt.cpu().numpy()[idx], ref, what=f"config {cfg}, {n} rays")
+
+
+def test_counts_where_rounding_decides_the_termination():
+    """A constant density makes every ray's transmittance after 20 samples the
+    same but for rounding, and the termination threshold is its median: the
+    order of the products decides the counts.  Cameras in every form and short
+    ray lists give the counts of the packed queue, which marches the same 8 x 4
+    tiles as a list of 2^14 rays."""
+    sc = synth.make_scene(1)
+    for k in ("grid", "p_xy", "p_xz", "p_yz"):
+        sc[k] = np.zeros_like(sc[k])
+    sc["grid"][..., 0] = 3.0
+    sc["occ"] = np.full_like(sc["occ"], 10.0) * np.array([-1.0, 1.0], np.float32)  # no ramp inside the box
+    w, h = 256, 64
+    cam = _camera(1, w, h)
+    rays = oracle.camera_rays(cam).reshape(h // 4, 4, w // 8, 8, 6).transpose(0, 2, 1, 3, 4).reshape(-1, 6)
+    rays = torch.as_tensor(np.ascontiguousarray(rays)).cuda()
+    # the queue's transmittances after exactly 20 samples (the saved training state)
+    _, saved, _ = om.train_fwd(gpu_scene(sc, t_thr=0.0, n_max=20), rays, torch.zeros(rays.shape[0], 3, device="cuda"))
+    state = saved.view(-1, 20)
+    after = state[state[:, 8].contiguous().view(torch.int32) == 20, 7]
+    scene = gpu_scene(sc, t_thr=float(after.median()))
+    rgb, cnt = om.render(scene, camera=cam)
+    _, queue = om.render(scene, rays=rays)  # 2^14 rays, 32 to a tile
+    tiled = queue.view(h // 4, w // 8, 4, 8).permute(0, 2, 1, 3).reshape(-1)
+    # the threshold does split the rays by rounding
+    assert (queue == 20).sum() >= 20 and (queue == 21).sum() >= 20
+    assert torch.equal(cnt, tiled)
+    for fill in (_camera(1, 512, 256), _camera(1, 1024, 1024)):
+        _, g = om.render_cameras(scene, [fill, cam])
+        assert torch.equal(g[-w * h:], tiled)
+    for n in (1, 40, 5000):
+        _, short = om.render(scene, rays=rays[:n].contiguous())
+        assert torch.equal(short, queue[:n])
