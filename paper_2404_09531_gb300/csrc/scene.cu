@@ -551,7 +551,7 @@ omerf_status omerf_scene_create(const omerf_scene_desc* desc, void* stream, omer
   s->device = dev;
   cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (s->num_sms < 1) s->num_sms = 1;
-  // OMERF_FAULT=alloc: the handle's first allocation fails (tests of the path)
+  // OMERF_FAULT=alloc: the handle's allocation fails (tests of the path)
   choose_coarse_level(s);
   size_t bytes[6];
   scene_alloc_bytes(desc, s->Mc, bytes);
