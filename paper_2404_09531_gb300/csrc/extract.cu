@@ -38,7 +38,7 @@ __device__ __forceinline__ int edges_below(float z0, float hz, int n, float z) {
     return EQUAL ? e <= z : e < z;
   };
   const float q = __fdividef(z - z0, hz);
-  const int guess = (int)fminf(fmaxf(q, 0.0f), (float)n) + 1 - SHIFT;  // (a NaN counts as 0)
+  const int guess = min((int)fminf(fmaxf(q, 0.0f), (float)n), n - 1 + SHIFT) + 1 - SHIFT;  // (a NaN counts as 0)
 #pragma unroll
   for (int t = 0; t < 2; t++) {
     const int c = min(max(guess - t, 0), n);
@@ -46,7 +46,7 @@ __device__ __forceinline__ int edges_below(float z0, float hz, int n, float z) {
   }
   int lo = 0, hi = n;
   while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
+    const int mid = lo + ((hi - lo) >> 1);
     if (below(mid)) lo = mid + 1;
     else hi = mid;
   }
@@ -63,24 +63,30 @@ __device__ __forceinline__ uint32_t range_word(int first, int last, int w) {
   return lo > hi ? 0u : (~0u << lo) & (~0u >> (31 - hi));
 }
 
-// A warp takes 32 columns (i, j .. j + 31), one per lane, and writes their W =
-// ceil(Nz / 32) words in order (bit b of word w is voxel k = 32 w + b).  A
+// A warp takes a unit: 32 consecutive columns (i, j), one per lane, and wc of
+// their W = ceil(Nz / 32) words (bit b of word w is voxel k = 32 w + b).  A
 // column that lies in one occupancy cell, the common case, has one interval,
-// found once; the words of a column that overlaps several cells are united
-// cell by cell.  Cell ranges are exact integer arithmetic, in 32 bits where
-// they fit (small).  Each block adds its voxel count once: an addition per
-// warp and word made the 16.8 M words of a 2048^2 x 128 grid queue for one
-// address (199 us, now 64 us; integer instructions bound it).
+// found once per unit; the words of a column that overlaps several cells are
+// united cell by cell.  Few tall columns are split into many units (wc < W).
+// Cell ranges are exact integer arithmetic, in 32 bits where they fit (small).
+// Each block adds its voxel count once: an addition per warp and word made the
+// 16.8 M words of a 2048^2 x 128 grid queue for one address (199 us, now 64 us;
+// integer instructions bound it).
+struct GridSplit {
+  long long cols;  // columns Nx Ny
+  int wc, chunks;  // words of a unit's columns, units per 32 columns
+  int small;
+};
+template <bool SPLIT>  // wc < W: a unit's words are not contiguous
 __global__ void __launch_bounds__(256) occupancy_grid_kernel(const float2* __restrict__ occ, int M, int Nx, int Ny,
-                                                            int Nz, float z0, float hz, int small,
+                                                            int Nz, float z0, float hz, const GridSplit g,
                                                             uint32_t* __restrict__ bits, unsigned long long* count) {
   __shared__ unsigned long long part[8];
-  const int W = (Nz + 31) >> 5, lane = threadIdx.x & 31;
-  const unsigned groups = ((unsigned)Ny + 31u) >> 5;  // of 32 columns in a row
-  const long long units = (long long)Nx * groups;
+  const int W = (int)(((unsigned)Nz + 31u) >> 5), lane = threadIdx.x & 31;
+  const long long units = ((g.cols + 31) >> 5) * (SPLIT ? g.chunks : 1);
   // cells [lo, hi] that voxel v of N along an axis overlaps
   auto cells = [&](int v, int N, int& lo, int& hi) {
-    if (small) {
+    if (g.small) {
       const unsigned a = (unsigned)v * (unsigned)M;
       lo = (int)(a / (unsigned)N);
       hi = (int)((a + (unsigned)M + (unsigned)N - 1u) / (unsigned)N) - 1;
@@ -91,38 +97,42 @@ __global__ void __launch_bounds__(256) occupancy_grid_kernel(const float2* __res
   };
   unsigned long long pop = 0;
   for (long long u = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); u < units; u += (long long)gridDim.x * 8) {
-    const int i = small ? (int)((unsigned)u / groups) : (int)(u / groups);
-    const int j0 = 32 * (int)(u - (long long)i * groups), j = j0 + lane;
-    int first = 1, last = 0, alo, ahi, blo = 0, bhi = -1;
-    cells(i, Nx, alo, ahi);
-    if (j < Ny) {
-      cells(j, Ny, blo, bhi);
+    const long long cg = SPLIT ? u / g.chunks : u;
+    const int w0 = SPLIT ? (int)(u - cg * g.chunks) * g.wc : 0;
+    const int wn = SPLIT ? min(g.wc, W - w0) : W;  // words of a column in this unit
+    const long long c0 = 32 * cg, c = c0 + lane;
+    int first = 1, last = 0, alo = 0, ahi = -1, blo = 0, bhi = -1;
+    if (c < g.cols) {
+      const int i = g.small ? (int)((unsigned)c / (unsigned)Ny) : (int)(c / Ny);
+      cells(i, Nx, alo, ahi);
+      cells((int)(c - (long long)i * Ny), Ny, blo, bhi);
       if (alo == ahi && blo == bhi) {
         const float2 z = __ldg(occ + (long long)alo * M + blo);
         if (z.x < z.y) voxel_range(z0, hz, Nz, z, first, last);
       }
     }
-    const bool several = __any_sync(kFull, blo <= bhi && (alo < ahi || blo < bhi));
-    const int words = min(32, Ny - j0) * W;
-    uint32_t* out = bits + ((long long)i * Ny + j0) * W;
+    const bool several = __any_sync(kFull, alo < ahi || blo < bhi);
+    const int words = (int)min(32ll, g.cols - c0) * wn;
+    uint32_t* out = bits + c0 * W + w0;
     for (int e0 = 0; e0 < words; e0 += 32) {
-      const int e = e0 + lane, col = min(e / W, 31), w = e - col * W;
+      const int e = e0 + lane, col = min(e / wn, 31), w = e - col * wn;
       const int f = __shfl_sync(kFull, first, col), l = __shfl_sync(kFull, last, col);
-      uint32_t word = range_word(f, l, w);
+      uint32_t word = range_word(f, l, w0 + w);
       if (several) {
+        const int a0 = __shfl_sync(kFull, alo, col), a1 = __shfl_sync(kFull, ahi, col);
         const int b0 = __shfl_sync(kFull, blo, col), b1 = __shfl_sync(kFull, bhi, col);
-        if (e < words && (alo < ahi || b0 < b1))
-          for (int a = alo; a <= ahi; a++)
+        if (e < words && (a0 < a1 || b0 < b1))
+          for (int a = a0; a <= a1; a++)
             for (int b = b0; b <= b1; b++) {
               const float2 z = __ldg(occ + (long long)a * M + b);
               int zf, zl;
               if (!(z.x < z.y)) continue;
               voxel_range(z0, hz, Nz, z, zf, zl);
-              word |= range_word(zf, zl, w);
+              word |= range_word(zf, zl, w0 + w);
             }
       }
       if (e < words) {
-        out[e] = word;
+        out[SPLIT ? (long long)col * W + w : e] = word;
         pop += __popc(word);
       }
     }
@@ -371,17 +381,29 @@ omerf_status omerf_occupancy_grid(const float aabb[6], const float* occ, int32_t
     set_error("occ must be 8-byte, bits 4-byte, count 8-byte aligned");
     return OMERF_EINVAL;
   }
-  const long long words = (long long)N[0] * N[1] * ((N[2] + 31) / 32);
+  const long long words = (long long)N[0] * N[1] * (((long long)N[2] + 31) / 32);
   if (words > (1LL << 40)) { set_error("occupancy grid too large"); return OMERF_ESHAPE; }
   const float hz = (aabb[5] - aabb[4]) / (float)N[2];
   if ((words + 255) / 256 > 0x7fffffffLL) { set_error("occupancy grid too large"); return OMERF_ESHAPE; }
   OMERF_LAUNCH_FAULT();
   omerf_status st = check_device_ptrs({{occ, "occ"}, {bits, "bits"}, {count, "count"}});
   if (st != OMERF_OK) return st;
-  const long long units = (long long)N[0] * ((N[1] + 31ll) / 32);
-  const int small = units < (1ll << 31) && ((long long)std::max(N[0], N[1]) + 1) * M + std::max(N[0], N[1]) < (1ll << 31);
-  occupancy_grid_kernel<<<grid_for(units, 8, 8 * sm_count()), 256, 0, (cudaStream_t)stream>>>(
-      reinterpret_cast<const float2*>(occ), M, N[0], N[1], N[2], aabb[4], hz, small, bits, count);
+  // Units: 32 whole columns, or so few of their words that every warp slot of
+  // the chip (64 per SM) has a unit, but not fewer than its lanes can share (us
+  // a call over a 256^2 plane with whole columns / split: 16 x 16 x 16384 voxels
+  // 12,090 / 192, 64 x 64 x 4096 479 / 66, one column of 2^22 38 s / 12 ms).
+  GridSplit g;
+  const int W = (int)(((long long)N[2] + 31) / 32), sms = sm_count();
+  g.cols = (long long)N[0] * N[1];
+  const long long groups = (g.cols + 31) / 32, split = std::max(1ll, 64ll * sms / groups);
+  const int fill = (int)((31 + std::min(32ll, g.cols)) / std::min(32ll, g.cols));  // words per column for 32 lanes
+  g.wc = (int)std::min<long long>({std::max<long long>((W + split - 1) / split, fill), W, 1ll << 20});
+  g.chunks = (W + g.wc - 1) / g.wc;
+  g.small = g.cols < (1ll << 31) &&
+            ((long long)std::max(N[0], N[1]) + 1) * M + std::max(N[0], N[1]) < (1ll << 31);
+  auto kern = g.chunks > 1 ? occupancy_grid_kernel<true> : occupancy_grid_kernel<false>;
+  kern<<<grid_for(groups * g.chunks, 8, 8 * sms), 256, 0, (cudaStream_t)stream>>>(
+      reinterpret_cast<const float2*>(occ), M, N[0], N[1], N[2], aabb[4], hz, g, bits, count);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OMERF_OK : cuda_fail(e, "occupancy grid launch");
 }
