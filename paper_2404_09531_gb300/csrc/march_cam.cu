@@ -118,12 +118,12 @@ __device__ __forceinline__ void mlp_units(const float* __restrict__ W, const flo
   }
 }
 
-// G(F, d) with the units of each layer spread over the G lanes of a ray (every
-// unit summed in the same order whatever G): all three outputs for G = 1,
-// output j in y[0] of lane j < 3 else.  sin and cos of 2, 4 and 8 d follow from
-// those of d by doubling (each doubling at most doubles the error: below 1e-6).
-// All lanes of the warp call it for G > 1.  The render of a 1080p frame spent
-// 0.39 of 2.83 ms here with twelve sincosf and one unit per FMA.
+// G(F, d) with the encoding's angles and the units of each layer spread over
+// the G lanes of a ray (every unit summed in the same order whatever G): all
+// three outputs for G = 1, output j in y[0] of lane j < 3 else.  Every sine and
+// cosine of the encoding is sincosf of its own angle, as in view_encoding:
+// doubling those of d is cheaper but loses a factor of ten at 8 d.  All lanes
+// of the warp call it for G > 1.
 template <int G>
 __device__ __forceinline__ void mlp_rays(const float* __restrict__ W, const float F[7], const float d[3], int j,
                                          float y[3]) {
@@ -131,19 +131,21 @@ __device__ __forceinline__ void mlp_rays(const float* __restrict__ W, const floa
   float x[34], h[N], a[16];
 #pragma unroll
   for (int i = 0; i < 7; i++) x[i] = F[i];
+  x[7] = d[0];
+  x[8] = d[1];
+  x[9] = d[2];
+  // angle 3 k + c is 2^k d_c: its sine is input 10 + 6 k + c, its cosine 13 + 6 k + c
+  float sn[(12 + G - 1) / G], cs[(12 + G - 1) / G];
 #pragma unroll
-  for (int c = 0; c < 3; c++) {
-    float s, co;
-    sincosf(d[c], &s, &co);
-    x[7 + c] = d[c];
+  for (int t = 0; t < (12 + G - 1) / G; t++) {
+    const int m = min(t * G + j, 11), k = m / 3, c = m - 3 * k;
+    sincosf((float)(1 << k) * (c == 0 ? d[0] : (c == 1 ? d[1] : d[2])), &sn[t], &cs[t]);
+  }
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-      x[10 + 6 * k + c] = s;
-      x[13 + 6 * k + c] = co;
-      const float s2 = 2.0f * s;
-      co = fmaf(-s2, s, 1.0f);
-      s = s2 * x[13 + 6 * k + c];
-    }
+  for (int m = 0; m < 12; m++) {
+    const int at = 10 + 6 * (m / 3) + m % 3;
+    x[at] = G == 1 ? sn[m / G] : __shfl_sync(kFull, sn[m / G], m % G, G);
+    x[at + 3] = G == 1 ? cs[m / G] : __shfl_sync(kFull, cs[m / G], m % G, G);
   }
   mlp_units<N, 34>(W + kTW1, W + kTB1, N * j, x, h);
 #pragma unroll
