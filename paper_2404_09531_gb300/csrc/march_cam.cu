@@ -222,18 +222,65 @@ __device__ __forceinline__ void transpose_lanes(float v[8], int j) {
   }
 }
 
+// The sums over a ray's samples are compensated: a ray's samples are taken one
+// after the other, where the packed queue's lane scans round a sample's
+// contribution about five times whatever the ray's length, and a plain sum
+// in order would be coarser (pixels of rays of 700 samples 3.7e-7 off 64-bit
+// ones instead of 1.8e-7, root mean square; with the compensation 1.6e-7.  It costs a 1080p frame 2 %).
+//
+// Transmittance T = h + l, the rounding errors of h's products carried along.
+struct Through {
+  float h = 1.0f, l = 0.0f;
+  __device__ __forceinline__ float value() const { return __fadd_rn(h, l); }
+  __device__ __forceinline__ void pass(float om) {  // through a sample with 1 - opacity om
+    const float p = __fmul_rn(h, om);
+    l = fmaf(l, om, fmaf(h, om, -p));
+    h = p;
+  }
+};
+// Kahan's sum s += w x with c the correction of the next term.
+__device__ __forceinline__ void add_to(float& s, float& c, float w, float x) {
+  const float y = fmaf(w, x, c), t = __fadd_rn(s, y);
+  c = __fsub_rn(y, __fsub_rn(t, s));
+  s = t;
+}
+// The same for two channels, packed (a - b as a + b (-1): one rounding).
+__device__ __forceinline__ void add_to2(float2& s, float2& c, float w, float x0, float x1) {
+  const float2 m = make_float2(-1.0f, -1.0f);
+  const float2 y = __ffma2_rn(make_float2(w, w), make_float2(x0, x1), c), t = __fadd2_rn(s, y);
+  c = __ffma2_rn(__ffma2_rn(s, m, t), m, y);
+  s = t;
+}
+
 // A ray's transmittance T carried through its G lanes' opacities in lane
-// order: returns the transmittance before this lane's sample; `last` is the
-// lane whose sample takes it below thr, G if none does.
+// order, in place: T becomes the transmittance before this lane's sample, or
+// after it (`after`); `last` is the lane whose sample takes it below thr, G if
+// none does.
 template <int G>
-__device__ __forceinline__ float chain(float T, float ah, bool hit, int j, int base, float thr, int& last) {
+__device__ __forceinline__ void chain(Through& T, Through& after, float ah, bool hit, int j, int base, float thr,
+                                      int& last) {
+  const float om = __fsub_rn(1.0f, ah);
+#pragma unroll
+  for (int i = 0; i < G - 1; i++) {
+    const float v = __shfl_sync(kFull, om, i, G);
+    if (i < j) T.pass(v);
+  }
+  after = T;
+  after.pass(om);
+  const unsigned below = hits_of<G>(hit && after.value() < thr, base);
+  last = below ? __ffs(below) - 1 : G;
+}
+// The same for the counted transmittance, with the products alone.
+template <int G>
+__device__ __forceinline__ float chain_counted(float T, float ah, bool hit, int j, int base, float thr, int& last) {
   const float om = __fsub_rn(1.0f, ah);
 #pragma unroll
   for (int i = 0; i < G - 1; i++) {
     const float v = __shfl_sync(kFull, om, i, G);
     if (i < j) T = __fmul_rn(T, v);
   }
-  const unsigned below = hits_of<G>(hit && __fmul_rn(T, om) < thr, base);
+  T = __fmul_rn(T, om);
+  const unsigned below = hits_of<G>(hit && T < thr, base);
   last = below ? __ffs(below) - 1 : G;
   return T;
 }
@@ -296,11 +343,12 @@ __device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, Warp
   if (valid && ((want >> lane) & 1u)) a.count[rid] = ws.s.cnt[lane];
 }
 
-// Resident CTAs per SM (1080p frame with 6, 7, 8 for G = 1: 2.55, 2.58, 2.58
-// ms; 640x360 with 6, 7 for G = 4: 455, 476 us; 320x180 with 6, 7 for G = 8:
-// 242, 208 us); the counting form keeps its second density sum in registers.
+// Resident CTAs per SM: a 1080p frame with 5, 6 for G = 1 2.35, 2.37 ms, with
+// counts (a second density sum in registers) with 4, 5 2.60, 2.94 ms; 641x361
+// with 5, 6 for G = 4 417, 434 us; 320x180 with 6, 7 for G = 8 242, 208 us;
+// 10,007 listed rays with counts with 4, 5 for G = 8 180, 144 us.
 template <class FT, bool SPARSE, int G, bool COUNT>
-__global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 ? 7 : 6))
+__global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 : 5) : (G == 8 ? 7 : 5))
     march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
   constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
   constexpr unsigned kFrameMask = (1u << kFrame) - 1u;
@@ -360,7 +408,14 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 
     unsigned wm = 0;
     bool need_mask = wb <= ke;
     bool amb = false, done = false, counted = false;
-    float T = 1.0f, Tc = 1.0f, F[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    Through T;
+    float Tc = 1.0f;
+    // the sums over the samples and their corrections: all channels for G = 1,
+    // channels j and j + 4 of lane j for G = 4 (in F2[0]), channel j for G = 8 (in F)
+    float2 F2[4], E2[4];
+    float F = 0.0f, E = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 4; c++) F2[c] = E2[c] = make_float2(0.0f, 0.0f);
     int seen = 0, cnt = 0;
     int k0 = 0;
     unsigned own = 0, todo = 0;
@@ -436,11 +491,11 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 
           activate(g, t, p[2], zb, s);
           seen++;
           if (!COUNT || !done) {
-            const float w = __fmul_rn(T, s.ah);
+            const float w = __fmul_rn(T.value(), s.ah);
 #pragma unroll
-            for (int c = 0; c < 7; c++) F[c] = fmaf(w, s.x[c], F[c]);
-            T = __fmul_rn(T, __fsub_rn(1.0f, s.ah));
-            done = T < g.t_thr;
+            for (int c = 0; c < 4; c++) add_to2(F2[c], E2[c], w, s.x[2 * c], c < 3 ? s.x[2 * c + 1] : 0.0f);
+            T.pass(__fsub_rn(1.0f, s.ah));
+            done = T.value() < g.t_thr;
           }
           if (COUNT && !counted) {
             t[0] = t0;
@@ -478,10 +533,11 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 
         if (!COUNT || __any_sync(kFull, !done)) {
           // transmittance before each lane's sample, in lattice order
           int last;
-          const float Ta = chain<G>(T, s.ah, hit, j, base, g.t_thr, last);
+          Through before = T, after;
+          chain<G>(before, after, s.ah, hit, j, base, g.t_thr, last);
           const unsigned kept = hits_of<G>(hit && !done && j <= last, base);
-          const float w = __fmul_rn(Ta, s.ah);
-          // lane j sums channels j and (G = 4) j + 4, sample after sample
+          const float w = __fmul_rn(before.value(), s.ah);
+          // lane j sums its channels, sample after sample
           float v[8];
 #pragma unroll
           for (int c = 0; c < 8; c++) v[c] = c < 7 ? s.x[c] : 0.0f;
@@ -490,17 +546,21 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 
           for (int i = 0; i < G; i++) {
             const float wi = __shfl_sync(kFull, w, i, G);
             if ((kept >> i) & 1u) {
-#pragma unroll
-              for (int r = 0; r < 8 / G; r++) F[r] = fmaf(wi, v[r * G + i], F[r]);
+              if (G == 4) add_to2(F2[0], E2[0], wi, v[i], v[(4 + i) & 7]);
+              else add_to(F, E, wi, v[i]);
             }
           }
-          const float Tn = __shfl_sync(kFull, __fmul_rn(Ta, __fsub_rn(1.0f, s.ah)), min(last, G - 1), G);
-          if (!done) T = Tn;
+          const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
+          const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
+          if (!done) {
+            T.h = th;
+            T.l = tl;
+          }
           done = done || last < G;
         }
         if (COUNT && __any_sync(kFull, !counted)) {
           int last;
-          const float Ta = __fmul_rn(chain<G>(Tc, ahc, hit, j, base, g.t_thr, last), __fsub_rn(1.0f, ahc));
+          const float Ta = chain_counted<G>(Tc, ahc, hit, j, base, g.t_thr, last);
           const bool kept = hit && !counted && j <= last;
           const int n = __popc(hits_of<G>(kept, base));
           if (!counted) cnt = seen + n;
@@ -520,25 +580,27 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? 5 : (G == 8 
     float out[3];
     if (G == 1) {
       if (valid) {
-        float yd[3] = {0.0f, 0.0f, 0.0f};
-        if (seen > 0) mlp_rays<1>(sW, F, d, 0, yd);
+        float yd[3] = {0.0f, 0.0f, 0.0f}, all[7];
 #pragma unroll
-        for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T, g.bg[c], F[c] + yd[c]) : g.bg[c];
+        for (int c = 0; c < 7; c++) all[c] = c & 1 ? F2[c / 2].y : F2[c / 2].x;
+        if (seen > 0) mlp_rays<1>(sW, all, d, 0, yd);
+#pragma unroll
+        for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T.value(), g.bg[c], all[c] + yd[c]) : g.bg[c];
 #pragma unroll
         for (int c = 0; c < 3; c++) a.rgb[3 * rid + c] = out[c];
         if (COUNT) a.count[rid] = cnt;
       }
     } else {
       float y[3] = {0.0f, 0.0f, 0.0f};
-      const float Fj = F[0];  // channel j
+      const float Fj = G == 4 ? F2[0].x : F;  // channel j
       if (__any_sync(kFull, seen > 0)) {
         float all[7];
 #pragma unroll
-        for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, F[c / G], c % G, G);
+        for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, c < G ? Fj : F2[0].y, c % G, G);
         mlp_rays<G>(sW, all, d, j, y);
       }
       if (valid && j < 3) {
-        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T, g.bg[j], Fj + y[0]) : g.bg[j];
+        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T.value(), g.bg[j], Fj + y[0]) : g.bg[j];
         if (COUNT && j == 0) a.count[rid] = cnt;
       }
     }
