@@ -33,8 +33,9 @@
 // ray's transmittance in different orders: where counts are wanted the
 // density is also summed in the queue's order, its transmittance decides the
 // count, and a ray that passes the termination threshold within the
-// products' rounding (about 1 of 10^5) is counted again by marching its
-// bundle with the queue.
+// products' rounding (1 of 10^5 in the city, 1 of 40 in fog of 0.01 per
+// sample) is counted again in the queue's order (see "Counts in the queue's
+// order").
 #include "march_fwd.cuh"
 
 namespace omerf {
@@ -313,34 +314,127 @@ __device__ __forceinline__ void load_ray(const float* __restrict__ r, float o[3]
   }
 }
 
-// March the 32 rays of one of the packed queue's bundles (an 8 x 4 tile, bit
-// 8 y + x, or 32 consecutive rays of a list) with the queue, and write the
-// sample counts of the rays whose bit is set in `want`.
-template <class FT, bool SPARSE, int G>
-__device__ __noinline__ void resolve_counts(const Geo& g, const FwdArgs& a, WarpMarch<false>& ws, unsigned sb, int t,
-                                            unsigned want) {
-  const int lane = threadIdx.x & 31;
-  bool valid;
-  long rid;
-  float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
-  if (a.use_cam) {
-    constexpr int kTilesX = (CamShape<G>::kW + 7) / 8;
-    int x0, y0;
-    long ray0;
-    const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
-    const int px = ((x0 >> 3) + t % kTilesX) * 8 + (lane & 7), py = ((y0 >> 2) + t / kTilesX) * 4 + (lane >> 3);
-    valid = px < cam.width && py < cam.height;
-    rid = ray0 + (long)py * cam.width + px;
-    if (valid) camera_ray(cam, px, py, o, d);
-  } else {
-    rid = ((long)sb * CamShape<G>::kRays & ~31l) + 32 * t + lane;
-    valid = rid < a.n;
-    if (valid) load_ray(a.rays + 6 * rid, o, d);
+// ---------------------------------------------------------------------------
+// Counts in the queue's order
+//
+// The queue takes a bundle's 32 rays (an 8 x 4 tile, bit 8 y + x, or 32
+// consecutive rays of a list) one after the other and fills 32 places at a
+// time with their evaluated samples; the transmittance of a ray's samples in a
+// batch is a lane scan from the ray's first place in it, so its rounding
+// depends on where the batches cut the ray and on nothing else.  The place
+// where a ray starts follows from the counts of the rays before it and from
+// whether their evaluated samples fill the batch they stop in (next_place).
+// So an ambiguous ray alone is marched again, 32 samples at a time by a warp,
+// and the other rays of its bundle only say how many samples they have beyond
+// their last one.  (Marching the whole bundle with the queue kept a CTA
+// waiting for one warp: a 333x201 city camera with one such ray took 560 us
+// instead of 225, 1280x720 pixels of fog of 0.01 per sample 48 ms, 15 without
+// counts.  Now 225 us and 17.5 ms.)
+// ---------------------------------------------------------------------------
+
+// Of the bundle's ray r: its count and its evaluated samples up to 31 beyond
+// the last counted one (or all of them); samples = -1: to be counted again.
+struct BundleCounts {
+  int count[32], samples[32];
+};
+
+// The queue's places filled after a ray that starts at `place`.
+__device__ __forceinline__ int next_place(int place, int count, int samples) {
+  const int free = 32 - place;
+  if (samples <= free) return (place + samples) & 31;  // all of them fit in
+  if (count <= free) return 0;                         // stopped in a batch that it filled
+  const int rest = (samples - free) - ((count - free - 1) & ~31);  // for the batch of its last sample
+  return rest >= 32 ? 0 : rest;
+}
+
+// A ray's evaluated samples after lattice index k, at most `want` (or a few
+// more), by its G lanes.  All lanes of the warp call it.
+template <int G>
+__device__ __noinline__ int samples_after(const Geo& g, float o0, float o1, float o2, float d0, float d1, float d2,
+                                          int k, int khi, int want, int j) {
+  const float o[3] = {o0, o1, o2}, d[3] = {d0, d1, d2};
+  int n = 0;
+#pragma unroll 1
+  for (int wb = k + 1; __any_sync(kFull, n < want && wb <= khi); wb += 1024) {
+    unsigned m = 0;
+    if (n < want)
+      for (int jw = j; jw < 32 && wb + 32 * jw <= khi; jw += G)
+        if (window_maybe(g, o, d, wb + 32 * jw, min(wb + 32 * jw + 31, khi))) m |= 1u << jw;
+#pragma unroll
+    for (int s = 1; s < G; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
+    while (__any_sync(kFull, n < want && m != 0u)) {
+      unsigned e = 0;
+      if (n < want && m != 0u) {
+        e = window_samples<G>(g, o, d, wb + 32 * (__ffs(m) - 1), k + 1, khi, j);
+        m &= m - 1u;
+      }
+#pragma unroll
+      for (int s = 1; s < G; s <<= 1) e |= __shfl_xor_sync(kFull, e, s);
+      n += __popc(e);
+    }
   }
-  int klo = 0, khi = -1;
-  const bool any = valid && lattice_range(g, o, d, klo, khi);
-  march_bundle<FT, SPARSE>(g, lane, o, d, klo, khi, any, ws);
-  if (valid && ((want >> lane) & 1u)) a.count[rid] = ws.s.cnt[lane];
+  return n;
+}
+
+// Count a ray (the same one in every lane) as the queue does from `place`, and
+// move `place` on.
+template <class FT, bool SPARSE>
+__device__ __forceinline__ int count_in_queue(const Geo& g, const float o[3], const float d[3], float4* sa, float* sb,
+                                              int lane, int& place) {
+  int klo = 0, khi = -1, count = 0, nq = place, first = place, taken = 0;
+  float T = 1.0f;
+  bool done = !lattice_range(g, o, d, klo, khi);
+  // the batch's places [first, nq): composite them
+  auto batch = [&]() {
+    __syncwarp();
+    const bool act = lane >= first && lane < nq;
+    SampleAct s;
+    s.ah = 0.0f;
+    if (act) {
+      const float4 q = sa[lane];
+      const float p[3] = {q.x, q.y, q.z};
+      float t[8];
+      gather_features<FT, SPARSE>(g, p, t);
+      activate(g, t, p[2], make_float2(q.w, sb[lane]), s);
+    }
+    const float Tn = T * seg_prod_scan(1.0f - s.ah, lane, first);
+    const unsigned below = __ballot_sync(kFull, act && Tn < g.t_thr);
+    count += below ? __ffs(below) - first : nq - first;
+    done = below != 0u;
+    T = __shfl_sync(kFull, Tn, nq - 1);
+    if (nq == 32) nq = 0;
+    first = nq;
+    __syncwarp();  // the places are read: they may be filled again
+  };
+  for (int wb = klo; !done && wb <= khi; wb += 1024) {
+    for (unsigned wm = window_mask(g, o, d, wb, khi, lane); wm && !done; wm &= wm - 1u) {
+      const int k = wb + 32 * (__ffs(wm) - 1) + lane;
+      float p[3];
+      float2 zb = make_float2(0.0f, 0.0f);
+      int cell = 0;
+      const bool ok = k <= khi && lattice_test(g, o, d, k, p, zb, cell);
+      for (unsigned m = __ballot_sync(kFull, ok); m && !done;) {
+        const int take = min(__popc(m), min(g.n_max - taken, 32 - nq)), rank = __popc(m & lanemask_lt());
+        const bool sel = ((m >> lane) & 1u) && rank < take;
+        if (sel) {
+          sa[nq + rank] = make_float4(p[0], p[1], p[2], zb.x);
+          sb[nq + rank] = zb.y;
+        }
+        m &= ~__ballot_sync(kFull, sel);
+        nq += take;
+        taken += take;
+        const bool last = taken >= g.n_max;
+        if (nq == 32) batch();
+        if (last) {
+          if (nq > first) batch();
+          done = true;
+        }
+      }
+    }
+  }
+  if (!done && nq > first) batch();
+  place = nq;
+  return count;
 }
 
 // Resident CTAs per SM: a 1080p frame with 5, 6 for G = 1 2.35, 2.37 ms, with
@@ -352,12 +446,14 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
     march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
   constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
   constexpr unsigned kFrameMask = (1u << kFrame) - 1u;
-  constexpr int kTilesX = (CamShape<G>::kW + 7) / 8, kTilesY = (CamShape<G>::kH + 3) / 4;
   __shared__ __align__(16) float sW[kSmemMlpT];
-  __shared__ typename std::conditional<COUNT, WarpMarch<false>, int>::type sMarch;
-  __shared__ unsigned sWork[2], sAmb[kTilesX * kTilesY];
+  // ambiguous counts: the bundles' rays and the places of a batch, per warp that replays
+  constexpr int kReplay = COUNT ? (G == 1 ? CamShape<G>::kWarps : 1) : 0;
+  __shared__ BundleCounts sCounts[kReplay > 0 ? kReplay : 1];
+  __shared__ float4 sQa[kReplay > 0 ? kReplay : 1][COUNT ? 32 : 1];
+  __shared__ float sQb[kReplay > 0 ? kReplay : 1][COUNT ? 32 : 1];
+  __shared__ unsigned sWork[2];
   load_mlp_units(g.mlp, sW);
-  if (COUNT && threadIdx.x < kTilesX * kTilesY) sAmb[threadIdx.x] = 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int base = lane & ~(kFrame - 1), j = G == 1 ? 0 : lane & (G - 1);
   // (without a counter there is one super-tile per CTA)
@@ -368,28 +464,28 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
     if (sb >= a.n_super) break;
     if (threadIdx.x == 0) sWork[it ^ 1] = a.counter ? atomicAdd(a.counter, 1u) : (unsigned)a.n_super;
 
+    // G = 8 with counts: half of one of the queue's bundles; if a ray of it is
+    // to be counted again, the other half is marched as well (for its counts)
+    for (int half = 0;; half++) {
     bool valid;
     long rid;
-    int amb_tile, amb_bit;  // the queue's bundle within the super-tile that holds this ray
+    int slot;  // the ray's place in its bundle
     float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
     if (a.use_cam) {
       int sx, sy, x0, y0;
       long ray0;
       lane_pixel<G>(warp, lane, sx, sy);
       const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
-      const int px = x0 + sx, py = y0 + sy;
+      const int px = (COUNT && G == 8 ? x0 ^ (4 * half) : x0) + sx, py = y0 + sy;
       valid = px < cam.width && py < cam.height;
       rid = ray0 + (long)py * cam.width + px;
       if (valid) camera_ray(cam, px, py, o, d);
-      amb_tile = (sy / 4) * kTilesX + sx / 8;
-      amb_bit = ((py & 3) << 3) | (px & 7);
+      slot = ((py & 3) << 3) | (px & 7);
     } else {
-      const int r = warp * (32 / G) + lane / G;
-      rid = (long)sb * CamShape<G>::kRays + r;
+      rid = (long)(COUNT && G == 8 ? sb ^ (unsigned)half : sb) * CamShape<G>::kRays + warp * (32 / G) + lane / G;
       valid = rid < a.n;
       if (valid) load_ray(a.rays + 6 * rid, o, d);
-      amb_tile = r >> 5;
-      amb_bit = (int)(rid & 31);
+      slot = (int)(rid & 31);
     }
     int klo = 0, khi = -1;
     bool alive = valid && lattice_range(g, o, d, klo, khi);
@@ -416,7 +512,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
     float F = 0.0f, E = 0.0f;
 #pragma unroll
     for (int c = 0; c < 4; c++) F2[c] = E2[c] = make_float2(0.0f, 0.0f);
-    int seen = 0, cnt = 0;
+    int seen = 0, cnt = 0, kstop = khi;  // kstop: the lattice index where the ray stopped
     int k0 = 0;
     unsigned own = 0, todo = 0;
     for (;;) {
@@ -465,6 +561,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
       // G = 1: the frame's next index, for the rays evaluated there; else the
       // ray's next G samples, one per lane
       unsigned left = todo;
+      const unsigned had = todo;
       if (G == 1) {
         todo &= todo - 1u;
       } else {
@@ -506,6 +603,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
             amb |= fabsf(Tc - g.t_thr) < g.t_thr * ambiguity(cnt);
           }
           alive = seen < g.n_max && !(done && (!COUNT || counted));
+          if (COUNT && !alive) kstop = k0 + bit;
         }
         const unsigned am = __ballot_sync(kFull, alive);
         if (((am >> base) & kFrameMask) == 0u) {
@@ -571,12 +669,14 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
         }
         seen += __popc(hits_of<G>(hit, base));
         if (seen >= g.n_max || (done && (!COUNT || counted))) {
+          if (COUNT && alive) kstop = k0 + 31 - __clz(had & ~todo);
           alive = need_mask = false;
           todo = wm = 0u;
         }
       }
     }
 
+    if (COUNT && G > 1) amb = hits_of<G>(amb, lane & ~(G - 1)) != 0u;
     float out[3];
     if (G == 1) {
       if (valid) {
@@ -588,9 +688,9 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
         for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T.value(), g.bg[c], all[c] + yd[c]) : g.bg[c];
 #pragma unroll
         for (int c = 0; c < 3; c++) a.rgb[3 * rid + c] = out[c];
-        if (COUNT) a.count[rid] = cnt;
+        if (COUNT && !amb) a.count[rid] = cnt;
       }
-    } else {
+    } else if (half == 0) {
       float y[3] = {0.0f, 0.0f, 0.0f};
       const float Fj = G == 4 ? F2[0].x : F;  // channel j
       if (__any_sync(kFull, seen > 0)) {
@@ -601,25 +701,60 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
       }
       if (valid && j < 3) {
         a.rgb[3 * rid + j] = seen > 0 ? fmaf(T.value(), g.bg[j], Fj + y[0]) : g.bg[j];
-        if (COUNT && j == 0) a.count[rid] = cnt;
+        if (COUNT && j == 0 && !amb) a.count[rid] = cnt;
       }
     }
-    if constexpr (COUNT) {
-      if (amb && valid) atomicOr(&sAmb[amb_tile], 1u << amb_bit);
-      __syncthreads();
-      if (warp == 0) {
-        // rays whose transmittance passed the termination threshold within
-        // rounding: count their tile's samples again
-#pragma unroll 1
-        for (int t = 0; t < kTilesX * kTilesY; t++) {
-          const unsigned want = sAmb[t];
-          if (want) {
-            resolve_counts<FT, SPARSE, G>(g, a, sMarch, sb, t, want);
-            __syncwarp();
-            if (lane == 0) sAmb[t] = 0u;
-          }
+    if constexpr (!COUNT) {
+      break;
+    } else {
+      // does a ray of the bundle have to be counted again?
+      if (G == 1 ? !__any_sync(kFull, amb) : !__syncthreads_or(amb) && half == 0) break;
+      BundleCounts& bc = sCounts[G == 1 ? warp : 0];
+      const int more = cnt + 31 - seen;  // wanted beyond the samples it has seen
+      const int extra = samples_after<G>(g, o[0], o[1], o[2], d[0], d[1], d[2], kstop, khi,
+                                         valid && seen < g.n_max && kstop < khi ? more : 0, j);
+      if (j == 0) {
+        bc.count[slot] = cnt;
+        bc.samples[slot] = amb ? -1 : min(min(seen + extra, g.n_max), cnt + 31);
+      }
+      if (G == 8 && half == 0) continue;
+      if (G == 1) __syncwarp();
+      else __syncthreads();
+      if (G != 1 && warp != 0) break;
+      int x0 = 0, y0 = 0, place = 0;
+      long ray0 = ((long)sb * CamShape<G>::kRays) & ~31l;
+      const Cam* cam = nullptr;
+      if (a.use_cam) {
+        cam = &tile_camera<G>(a, sb, x0, y0, ray0);
+        if (G == 1) {
+          x0 += (warp & 1) * 8;
+          y0 += (warp >> 1) * 4;
         }
       }
+#pragma unroll 1
+      for (unsigned again = __ballot_sync(kFull, bc.samples[lane] < 0), r = 0; r < 32 && again >> r; r++) {
+        if (!((again >> r) & 1u)) {
+          place = next_place(place, bc.count[r], bc.samples[r]);
+        } else {
+          // (a ray of the other half is counted for its place only)
+          float ro[3], rd[3];
+          bool own = true;
+          long id = ray0 + r;
+          if (a.use_cam) {
+            const int px = (x0 & ~7) + (r & 7), py = y0 + (r >> 3);
+            own = G != 8 || ((px ^ x0) & 4) == 0;
+            id = ray0 + (long)py * cam->width + px;
+            camera_ray(*cam, px, py, ro, rd);
+          } else {
+            own = G != 8 || (r >> 4) == (sb & 1u);
+            load_ray(a.rays + 6 * id, ro, rd);
+          }
+          const int n = count_in_queue<FT, SPARSE>(g, ro, rd, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0], lane, place);
+          if (own && lane == 0) a.count[id] = n;
+        }
+      }
+      break;
+    }
     }
     __syncthreads();
   }
