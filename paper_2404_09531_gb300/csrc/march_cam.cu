@@ -239,17 +239,18 @@ struct Through {
     h = p;
   }
 };
-// Kahan's sum s += w x with c the correction of the next term.
+// A sum s + c of terms w x: the error of every sum is the term less what it
+// changed s by, added up in c beside the chain of s.
 __device__ __forceinline__ void add_to(float& s, float& c, float w, float x) {
-  const float y = fmaf(w, x, c), t = __fadd_rn(s, y);
-  c = __fsub_rn(y, __fsub_rn(t, s));
+  const float t = fmaf(w, x, s);
+  c = __fadd_rn(c, fmaf(w, x, __fsub_rn(s, t)));
   s = t;
 }
-// The same for two channels, packed (a - b as a + b (-1): one rounding).
+// The same for two channels, packed (s - t as t (-1) + s: one rounding).
 __device__ __forceinline__ void add_to2(float2& s, float2& c, float w, float x0, float x1) {
-  const float2 m = make_float2(-1.0f, -1.0f);
-  const float2 y = __ffma2_rn(make_float2(w, w), make_float2(x0, x1), c), t = __fadd2_rn(s, y);
-  c = __ffma2_rn(__ffma2_rn(s, m, t), m, y);
+  const float2 ww = make_float2(w, w), x = make_float2(x0, x1);
+  const float2 t = __ffma2_rn(ww, x, s);
+  c = __fadd2_rn(c, __ffma2_rn(ww, x, __ffma2_rn(t, make_float2(-1.0f, -1.0f), s)));
   s = t;
 }
 
@@ -682,7 +683,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
       if (valid) {
         float yd[3] = {0.0f, 0.0f, 0.0f}, all[7];
 #pragma unroll
-        for (int c = 0; c < 7; c++) all[c] = c & 1 ? F2[c / 2].y : F2[c / 2].x;
+        for (int c = 0; c < 7; c++) all[c] = c & 1 ? F2[c / 2].y + E2[c / 2].y : F2[c / 2].x + E2[c / 2].x;
         if (seen > 0) mlp_rays<1>(sW, all, d, 0, yd);
 #pragma unroll
         for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T.value(), g.bg[c], all[c] + yd[c]) : g.bg[c];
@@ -692,11 +693,11 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
       }
     } else if (half == 0) {
       float y[3] = {0.0f, 0.0f, 0.0f};
-      const float Fj = G == 4 ? F2[0].x : F;  // channel j
+      const float Fj = G == 4 ? F2[0].x + E2[0].x : F + E;  // channel j
       if (__any_sync(kFull, seen > 0)) {
         float all[7];
 #pragma unroll
-        for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, c < G ? Fj : F2[0].y, c % G, G);
+        for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, c < G ? Fj : F2[0].y + E2[0].y, c % G, G);
         mlp_rays<G>(sW, all, d, j, y);
       }
       if (valid && j < 3) {
