@@ -31,11 +31,11 @@
 // Sample counts are those of the packed queue, which training and long ray
 // lists use, also where rounding decides them.  The two forms multiply a
 // ray's transmittance in different orders: where counts are wanted the
-// density is also summed in the queue's order, its transmittance decides the
-// count, and a ray that passes the termination threshold within the
-// products' rounding (1 of 10^5 in the city, 1 of 40 in fog of 0.01 per
-// sample) is counted again in the queue's order (see "Counts in the queue's
-// order").
+// density is also summed in the queue's order, its transmittance (compensated,
+// so that the queue's rounding alone is in doubt) decides the count, and a ray
+// that passes the termination threshold within that rounding (1 of 2 x 10^5 in
+// the city, 1 of 80 in fog of 0.01 per sample) is counted again in the queue's
+// order (see "Counts in the queue's order").
 #include "march_fwd.cuh"
 
 namespace omerf {
@@ -272,21 +272,6 @@ __device__ __forceinline__ void chain(Through& T, Through& after, float ah, bool
   const unsigned below = hits_of<G>(hit && after.value() < thr, base);
   last = below ? __ffs(below) - 1 : G;
 }
-// The same for the counted transmittance, with the products alone.
-template <int G>
-__device__ __forceinline__ float chain_counted(float T, float ah, bool hit, int j, int base, float thr, int& last) {
-  const float om = __fsub_rn(1.0f, ah);
-#pragma unroll
-  for (int i = 0; i < G - 1; i++) {
-    const float v = __shfl_sync(kFull, om, i, G);
-    if (i < j) T = __fmul_rn(T, v);
-  }
-  T = __fmul_rn(T, om);
-  const unsigned below = hits_of<G>(hit && T < thr, base);
-  last = below ? __ffs(below) - 1 : G;
-  return T;
-}
-
 // The camera of super-tile sb, its pixel origin and first ray.
 template <int G>
 __device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb, int& x0, int& y0, long& ray0) {
@@ -330,7 +315,7 @@ __device__ __forceinline__ void load_ray(const float* __restrict__ r, float o[3]
 // their last one.  (Marching the whole bundle with the queue kept a CTA
 // waiting for one warp: a 333x201 city camera with one such ray took 560 us
 // instead of 225, 1280x720 pixels of fog of 0.01 per sample 48 ms, 15 without
-// counts.  Now 225 us and 17.5 ms.)
+// counts.  Now 225 us and 17.1 ms.)
 // ---------------------------------------------------------------------------
 
 // Of the bundle's ray r: its count and its evaluated samples up to 31 beyond
@@ -505,8 +490,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
     unsigned wm = 0;
     bool need_mask = wb <= ke;
     bool amb = false, done = false, counted = false;
-    Through T;
-    float Tc = 1.0f;
+    Through T, Tc;  // of the pixel's densities and of the counts'
     // the sums over the samples and their corrections: all channels for G = 1,
     // channels j and j + 4 of lane j for G = 4 (in F2[0]), channel j for G = 8 (in F)
     float2 F2[4], E2[4];
@@ -598,10 +582,10 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
           if (COUNT && !counted) {
             t[0] = t0;
             activate(g, t, p[2], zb, s);
-            Tc = __fmul_rn(Tc, __fsub_rn(1.0f, s.ah));
+            Tc.pass(__fsub_rn(1.0f, s.ah));
             cnt = seen;
-            counted = Tc < g.t_thr;
-            amb |= fabsf(Tc - g.t_thr) < g.t_thr * ambiguity(cnt);
+            counted = Tc.value() < g.t_thr;
+            amb |= fabsf(Tc.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
           }
           alive = seen < g.n_max && !(done && (!COUNT || counted));
           if (COUNT && !alive) kstop = k0 + bit;
@@ -659,13 +643,18 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
         }
         if (COUNT && __any_sync(kFull, !counted)) {
           int last;
-          const float Ta = chain_counted<G>(Tc, ahc, hit, j, base, g.t_thr, last);
+          Through before = Tc, after;
+          chain<G>(before, after, ahc, hit, j, base, g.t_thr, last);
           const bool kept = hit && !counted && j <= last;
           const int n = __popc(hits_of<G>(kept, base));
           if (!counted) cnt = seen + n;
-          amb |= kept && fabsf(Ta - g.t_thr) < g.t_thr * ambiguity(cnt);
-          const float Tn = __shfl_sync(kFull, Ta, min(last, G - 1), G);
-          if (!counted) Tc = Tn;
+          amb |= kept && fabsf(after.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
+          const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
+          const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
+          if (!counted) {
+            Tc.h = th;
+            Tc.l = tl;
+          }
           counted = counted || last < G;
         }
         seen += __popc(hits_of<G>(hit, base));

@@ -129,9 +129,10 @@ struct FwdArgs {
 };
 
 // Relative distance from the termination threshold within which the order of
-// the transmittance's products could decide a sample: each of the two orders
-// rounds at most cnt products (2^-24 each).
-__device__ __forceinline__ float ambiguity(int cnt) { return 1e-6f + 1.3e-7f * (float)cnt; }
+// the transmittance's products could decide a sample: the queue rounds at most
+// cnt products by 2^-24 each, march_cam.cu's own transmittance (compensated)
+// is good to two roundings.  The factors are the same in both.
+__device__ __forceinline__ float ambiguity(int cnt) { return 2.5e-7f + 6.2e-8f * (float)cnt; }
 
 // Camera render with `lanes` lanes per ray (march_cam.cu).
 cudaError_t launch_render_cam(const omerf_scene* s, const FwdArgs& a, int lanes, cudaStream_t stream);
