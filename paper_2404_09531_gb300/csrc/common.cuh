@@ -651,14 +651,17 @@ struct SampleAct {
   float r;
 };
 
+// (pinned: a sample's opacity and 1 - opacity are the same bits in every kernel,
+// whatever it is inlined into, and the sample counts of all forms rest on that)
 __device__ __forceinline__ void activate(const Geo& g, const float t[8], float z, float2 zb, SampleAct& s) {
   s.Mv = occupancy(g, z, zb, s.branch, s.r);
   const float tau = __expf(t[0]);
   s.sigma = tau * g.step;
   // 1 - exp(-sigma): series for small sigma keeps the relative accuracy of alpha
-  s.alpha = s.sigma < 1e-3f ? s.sigma * (1.0f - 0.5f * s.sigma * (1.0f - s.sigma * (1.0f / 3.0f)))
-                            : 1.0f - __expf(-s.sigma);
-  s.ah = s.Mv * s.alpha;
+  s.alpha = s.sigma < 1e-3f
+                ? __fmul_rn(s.sigma, fmaf(__fmul_rn(-0.5f, s.sigma), fmaf(-s.sigma, 1.0f / 3.0f, 1.0f), 1.0f))
+                : __fsub_rn(1.0f, __expf(-s.sigma));
+  s.ah = __fmul_rn(s.Mv, s.alpha);
 #pragma unroll
   for (int c = 0; c < 7; c++) s.x[c] = sigmoid_fast(t[c + 1]);
 }

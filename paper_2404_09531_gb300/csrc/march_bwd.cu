@@ -591,7 +591,7 @@ __device__ __forceinline__ void march_bundle_bwd(const Geo& g, const BwdArgs& a,
     }
     bool head;
     const int segstart = segment_start(lane, r, head);
-    const float P = seg_prod_scan(1.0f - s.ah, lane, segstart);
+    const float P = seg_prod_scan(__fsub_rn(1.0f, s.ah), lane, segstart);
     float Pex = __shfl_up_sync(kFull, P, 1);
     if (head) Pex = 1.0f;
     const float Tprev = act ? ws.T[r] : 1.0f;

@@ -383,7 +383,7 @@ __device__ __forceinline__ int count_in_queue(const Geo& g, const float o[3], co
       gather_features<FT, SPARSE>(g, p, t);
       activate(g, t, p[2], make_float2(q.w, sb[lane]), s);
     }
-    const float Tn = T * seg_prod_scan(1.0f - s.ah, lane, first);
+    const float Tn = T * seg_prod_scan(__fsub_rn(1.0f, s.ah), lane, first);
     const unsigned below = __ballot_sync(kFull, act && Tn < g.t_thr);
     count += below ? __ffs(below) - first : nq - first;
     done = below != 0u;

@@ -74,7 +74,7 @@ __device__ __forceinline__ void march_bundle(const Geo& g, int lane, const float
     bool head;
     const int segstart = segment_start(lane, r, head);
     // transmittance: segmented inclusive product scan of (1 - alpha_hat)
-    const float P = seg_prod_scan(1.0f - s.ah, lane, segstart);
+    const float P = seg_prod_scan(__fsub_rn(1.0f, s.ah), lane, segstart);
     float Pex = __shfl_up_sync(kFull, P, 1);
     if (head) Pex = 1.0f;
     const float Tprev = act ? ws.s.T[r] : 1.0f;

@@ -99,3 +99,30 @@ def test_counting_costs_little_in_fog():
         return min(times)
 
     assert fastest(True) <= 2 * fastest(False)
+
+
+def test_counts_of_opaque_samples_in_ramps():
+    """Occupancy ramps over most of the box and opacities near 1, where a factor
+    rounded another way would move the transmittance most: thresholds at the
+    queue's own transmittances after two samples, and one step beside them."""
+    sc = synth.make_scene(1)
+    sc["grid"][..., 0] = np.random.default_rng(5).uniform(np.log(256 * 0.5), np.log(256 * 12), sc["grid"].shape[:3])
+    for k in ("p_xy", "p_xz", "p_yz"):
+        sc[k][..., 0] = 0.0
+    sc["occ"] = np.full_like(sc["occ"], 0.12) * np.array([-1.0, 1.0], np.float32)
+    rng = np.random.default_rng(6)
+    n = 1 << 14
+    o = rng.uniform(-0.9, 0.9, (n, 3)) * np.array([1.0, 1.0, 0.1])
+    d = rng.normal(size=(n, 3))
+    rays = torch.as_tensor(np.concatenate([o, d / np.linalg.norm(d, axis=1, keepdims=True)], 1).astype(np.float32)).cuda()
+    _, saved, _ = om.train_fwd(gpu_scene(sc, eps=0.12, n_max=2, t_thr=0.0), rays, torch.zeros(n, 3, device="cuda"))
+    T = saved.view(-1, 20)[:8192, 7]
+    T = T[(T > 1e-4) & (T < 0.3)].sort().values
+    assert T.numel() > 1000
+    for q in np.linspace(0, T.numel() - 1, 8).astype(int):
+        t = np.float32(T[int(q)].item())
+        for thr in (np.nextafter(t, np.float32(0)), t, np.nextafter(t, np.float32(1))):
+            scene = gpu_scene(sc, eps=0.12, t_thr=float(thr))
+            _, queue = om.render(scene, rays=rays)
+            _, short = om.render(scene, rays=rays[:8192].contiguous())
+            assert torch.equal(short, queue[:8192])
