@@ -68,11 +68,11 @@ struct Cam {
 };
 
 // One camera of a multi-camera render: its first super-tile and first ray
-// in the launch's numbering, and its super-tiles per row.
+// in the launch's numbering, its super-tiles per row and their form.
 struct CamRec {
   Cam cam;
   long long super_start, ray_start;
-  int super_x, pad;
+  int super_x, lw;
 };
 constexpr int kMaxCams = 16;  // cameras per multi-camera launch
 

@@ -76,6 +76,54 @@ __device__ __forceinline__ void lane_pixel(int warp, int lane, int& x, int& y) {
   }
 }
 
+// Images of one or two rows, or of up to four columns (two for G = 8), would
+// leave most pixels of such a super-tile empty.  They are cut into sub-tiles of
+// 2^lw columns with as many rays as a CTA (G = 4, 8) or a warp (G = 1) takes,
+// which holds whole 8 x 4 bundles of the queue, as far as the image has pixels
+// there: ray i is the pixel at place i of the bundles' pixels, one bundle after
+// the other.  (us, city pixels in one column / row with the queue, plain
+// super-tiles and these: 900,000 pixels 2782 / 4798, 8368 / 6502, 824 / 1326;
+// 60,000 pixels 212 / 376, 278 / 409, 131 / 194.)
+struct SubTile {
+  int lw, lbw, lbh;  // log2 of the width, and of the bundles' width and height in the image
+  template <int G>
+  static constexpr int kLog = G == 8 ? 4 : 5;
+};
+template <int G>
+__device__ __forceinline__ SubTile sub_tile(int lw) {
+  return {lw, min(lw, 3), min(SubTile::kLog<G> - lw, 2)};
+}
+__device__ __forceinline__ void sub_pixel(const SubTile& t, int i, int& x, int& y) {
+  const int b = i >> (t.lbw + t.lbh), w = i & ((1 << (t.lbw + t.lbh)) - 1), lnx = t.lw - t.lbw;
+  x = ((b & ((1 << lnx) - 1)) << t.lbw) + (w & ((1 << t.lbw) - 1));
+  y = ((b >> lnx) << t.lbh) + (w >> t.lbw);
+}
+// Origin of a warp's sub-tile (G = 1: four of them, along the image) in its super-tile.
+template <int G>
+__device__ __forceinline__ void sub_origin(int lw, int warp, int& x, int& y) {
+  if (G != 1) return;
+  if (lw < 0) {
+    x += (warp & 1) * 8;
+    y += (warp >> 1) * 4;
+  } else if (lw < 3) {
+    y += warp * (32 >> lw);
+  } else {
+    x += warp << lw;
+  }
+}
+
+// The pixels of a super-tile.
+static __host__ __device__ __forceinline__ void super_size(int lanes, int lw, int& w, int& h) {
+  if (lw < 0) {
+    w = lanes == 1 ? CamShape<1>::kW : (lanes == 4 ? CamShape<4>::kW : CamShape<8>::kW);
+    h = lanes == 1 ? CamShape<1>::kH : (lanes == 4 ? CamShape<4>::kH : CamShape<8>::kH);
+  } else {
+    w = 1 << lw;
+    h = (lanes == 8 ? 16 : 32) >> lw;
+    if (lanes == 1) (lw < 3 ? h : w) *= 4;
+  }
+}
+
 // The deferred MLP's weights with the units of a layer as the fast axis, so that
 // two units share one packed FMA: W1 [34][16], b1 [16], W2 [16][16], b2 [16],
 // W3 [16][4 (3 used)], b3 [4 (3 used)].
@@ -272,11 +320,13 @@ __device__ __forceinline__ void chain(Through& T, Through& after, float ah, bool
   const unsigned below = hits_of<G>(hit && after.value() < thr, base);
   last = below ? __ffs(below) - 1 : G;
 }
-// The camera of super-tile sb, its pixel origin and first ray.
+// The camera of super-tile sb, its form (see SubTile), pixel origin and first ray.
 template <int G>
-__device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb, int& x0, int& y0, long& ray0) {
+__device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb, int& lw, int& x0, int& y0,
+                                                  long& ray0) {
   const Cam* cam = &a.cam;
   int super_x = a.super_x;
+  lw = a.lw;
   ray0 = 0;
   if (a.n_cams > 0) {
     int c = 0;
@@ -285,10 +335,13 @@ __device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb,
     sb = (unsigned)((long long)sb - cr.super_start);
     cam = &cr.cam;
     super_x = cr.super_x;
+    lw = cr.lw;
     ray0 = (long)cr.ray_start;
   }
-  x0 = (int)(sb % (unsigned)super_x) * CamShape<G>::kW;
-  y0 = (int)(sb / (unsigned)super_x) * CamShape<G>::kH;
+  int w, h;
+  super_size(G, lw, w, h);
+  x0 = (int)(sb % (unsigned)super_x) * w;
+  y0 = (int)(sb / (unsigned)super_x) * h;
   return *cam;
 }
 
@@ -423,6 +476,61 @@ __device__ __forceinline__ int count_in_queue(const Geo& g, const float o[3], co
   return count;
 }
 
+template <int G>
+__device__ __noinline__ bool whole_bundles(const FwdArgs& a, unsigned sb) {
+  int lw, x0, y0;
+  long ray0;
+  tile_camera<G>(a, sb, lw, x0, y0, ray0);
+  return lw >= 0;
+}
+
+// Count the ambiguous rays of a warp's (G = 1) or a CTA's bundles, and write
+// their counts (a call of its own, so that the march keeps its registers).
+template <class FT, bool SPARSE, int G>
+__device__ __noinline__ void count_again(const Geo& g, const FwdArgs& a, unsigned sb, int warp, const BundleCounts& bc,
+                                         float4* qa, float* qb) {
+  const int lane = threadIdx.x & 31;
+  int lw = -1, x0 = 0, y0 = 0, place = 0;
+  long ray0 = ((long)sb * CamShape<G>::kRays) & ~31l;
+  const Cam* cam = nullptr;
+  if (a.use_cam) {
+    cam = &tile_camera<G>(a, sb, lw, x0, y0, ray0);
+    sub_origin<G>(lw, warp, x0, y0);
+  }
+  const SubTile st = sub_tile<G>(max(lw, 0));
+  const unsigned starts = lw < 0 ? 0u : (1u << (st.lbw + st.lbh)) - 1u;  // of bundles: r & starts == 0
+  unsigned again = __ballot_sync(kFull, bc.samples[lane] < 0);
+  if (G == 8 && lw >= 0) again &= 0xffffu;  // (the other half of the places is not in use)
+#pragma unroll 1
+  for (unsigned r = 0; r < 32 && again >> r; r++) {
+    if (starts && (r & starts) == 0u) place = 0;
+    if (!((again >> r) & 1u)) {
+      place = next_place(place, bc.count[r], bc.samples[r]);
+      continue;
+    }
+    // (a ray of the other half is counted for its place only)
+    float o[3], d[3];
+    bool own = true;
+    long id = ray0 + r;
+    if (a.use_cam) {
+      int px = (x0 & ~7) + (r & 7), py = y0 + (r >> 3);
+      if (lw >= 0) {
+        sub_pixel(st, r, px, py);
+        px += x0;
+        py += y0;
+      }
+      own = G != 8 || lw >= 0 || ((px ^ x0) & 4) == 0;
+      id = ray0 + (long)py * cam->width + px;
+      camera_ray(*cam, px, py, o, d);
+    } else {
+      own = G != 8 || (r >> 4) == (sb & 1u);
+      load_ray(a.rays + 6 * id, o, d);
+    }
+    const int n = count_in_queue<FT, SPARSE>(g, o, d, qa, qb, lane, place);
+    if (own && lane == 0) a.count[id] = n;
+  }
+}
+
 // Resident CTAs per SM: a 1080p frame with 5, 6 for G = 1 2.35, 2.37 ms, with
 // counts (a second density sum in registers) with 4, 5 2.60, 2.94 ms; 641x361
 // with 5, 6 for G = 4 417, 434 us; 320x180 with 6, 7 for G = 8 242, 208 us;
@@ -453,298 +561,276 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
     // G = 8 with counts: half of one of the queue's bundles; if a ray of it is
     // to be counted again, the other half is marched as well (for its counts)
     for (int half = 0;; half++) {
-    bool valid;
-    long rid;
-    int slot;  // the ray's place in its bundle
-    float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
-    if (a.use_cam) {
-      int sx, sy, x0, y0;
-      long ray0;
-      lane_pixel<G>(warp, lane, sx, sy);
-      const Cam& cam = tile_camera<G>(a, sb, x0, y0, ray0);
-      const int px = (COUNT && G == 8 ? x0 ^ (4 * half) : x0) + sx, py = y0 + sy;
-      valid = px < cam.width && py < cam.height;
-      rid = ray0 + (long)py * cam.width + px;
-      if (valid) camera_ray(cam, px, py, o, d);
-      slot = ((py & 3) << 3) | (px & 7);
-    } else {
-      rid = (long)(COUNT && G == 8 ? sb ^ (unsigned)half : sb) * CamShape<G>::kRays + warp * (32 / G) + lane / G;
-      valid = rid < a.n;
-      if (valid) load_ray(a.rays + 6 * rid, o, d);
-      slot = (int)(rid & 31);
-    }
-    int klo = 0, khi = -1;
-    bool alive = valid && lattice_range(g, o, d, klo, khi);
-    if (!alive) {
-      klo = 0x7fffffff;
-      khi = -1;
-    }
-    // the common lattice frame and its blocks of 32 windows from wb
-    int wb = klo, ke = khi;
-    if (G == 1) {
-      wb = min(wb, __shfl_xor_sync(kFull, wb, 1));
-      wb = min(wb, __shfl_xor_sync(kFull, wb, 2));
-      ke = max(ke, __shfl_xor_sync(kFull, ke, 1));
-      ke = max(ke, __shfl_xor_sync(kFull, ke, 2));
-    }
-    unsigned wm = 0;
-    bool need_mask = wb <= ke;
-    bool amb = false, done = false, counted = false;
-    Through T, Tc;  // of the pixel's densities and of the counts'
-    // the sums over the samples and their corrections: all channels for G = 1,
-    // channels j and j + 4 of lane j for G = 4 (in F2[0]), channel j for G = 8 (in F)
-    float2 F2[4], E2[4];
-    float F = 0.0f, E = 0.0f;
+      bool valid;
+      long rid;
+      int slot;  // the ray's place in its bundle
+      float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
+      if (a.use_cam) {
+        int px, py, lw, x0, y0;
+        long ray0;
+        const Cam& cam = tile_camera<G>(a, sb, lw, x0, y0, ray0);
+        if (lw < 0) {
+          lane_pixel<G>(warp, lane, px, py);
+          px += COUNT && G == 8 ? x0 ^ (4 * half) : x0;
+          py += y0;
+          slot = ((py & 3) << 3) | (px & 7);
+        } else {
+          slot = G == 1 ? lane : warp * (32 / G) + lane / G;
+          sub_pixel(sub_tile<G>(lw), slot, px, py);
+          sub_origin<G>(lw, warp, x0, y0);
+          px += x0;
+          py += y0;
+        }
+        valid = px < cam.width && py < cam.height;
+        rid = ray0 + (long)py * cam.width + px;
+        if (valid) camera_ray(cam, px, py, o, d);
+      } else {
+        rid = (long)(COUNT && G == 8 ? sb ^ (unsigned)half : sb) * CamShape<G>::kRays + warp * (32 / G) + lane / G;
+        valid = rid < a.n;
+        if (valid) load_ray(a.rays + 6 * rid, o, d);
+        slot = (int)(rid & 31);
+      }
+      int klo = 0, khi = -1;
+      bool alive = valid && lattice_range(g, o, d, klo, khi);
+      if (!alive) {
+        klo = 0x7fffffff;
+        khi = -1;
+      }
+      // the common lattice frame and its blocks of 32 windows from wb
+      int wb = klo, ke = khi;
+      if (G == 1) {
+        wb = min(wb, __shfl_xor_sync(kFull, wb, 1));
+        wb = min(wb, __shfl_xor_sync(kFull, wb, 2));
+        ke = max(ke, __shfl_xor_sync(kFull, ke, 1));
+        ke = max(ke, __shfl_xor_sync(kFull, ke, 2));
+      }
+      unsigned wm = 0;
+      bool need_mask = wb <= ke;
+      bool amb = false, done = false, counted = false;
+      Through T, Tc;  // of the pixel's densities and of the counts'
+      // the sums over the samples and their corrections: all channels for G = 1,
+      // channels j and j + 4 of lane j for G = 4 (in F2[0]), channel j for G = 8 (in F)
+      float2 F2[4], E2[4];
+      float F = 0.0f, E = 0.0f;
 #pragma unroll
-    for (int c = 0; c < 4; c++) F2[c] = E2[c] = make_float2(0.0f, 0.0f);
-    int seen = 0, cnt = 0, kstop = khi;  // kstop: the lattice index where the ray stopped
-    int k0 = 0;
-    unsigned own = 0, todo = 0;
-    for (;;) {
-      // A frame whose window is done takes its next one that the coarse grid
-      // cannot rule out.  With one lane per ray the frames of a warp do so
-      // together (a window is 32 tests for every lane), else each when it has to.
-      if (G > 1 || !__any_sync(kFull, todo != 0u)) {
-        while (__any_sync(kFull, todo == 0u && need_mask)) {
-          const bool now = todo == 0u && need_mask;
-          unsigned m = 0;
-          if (now && alive) {
-            const int nw = min((ke - wb) >> 5, 31);
-            for (int jw = j; jw <= nw; jw += G) {
-              const int ka = max(wb + 32 * jw, klo), kz = min(wb + 32 * jw + 31, khi);
-              if (ka <= kz && window_maybe(g, o, d, ka, kz)) m |= 1u << jw;
+      for (int c = 0; c < 4; c++) F2[c] = E2[c] = make_float2(0.0f, 0.0f);
+      int seen = 0, cnt = 0, kstop = khi;  // kstop: the lattice index where the ray stopped
+      int k0 = 0;
+      unsigned own = 0, todo = 0;
+      for (;;) {
+        // A frame whose window is done takes its next one that the coarse grid
+        // cannot rule out.  With one lane per ray the frames of a warp do so
+        // together (a window is 32 tests for every lane), else each when it has to.
+        if (G > 1 || !__any_sync(kFull, todo != 0u)) {
+          while (__any_sync(kFull, todo == 0u && need_mask)) {
+            const bool now = todo == 0u && need_mask;
+            unsigned m = 0;
+            if (now && alive) {
+              const int nw = min((ke - wb) >> 5, 31);
+              for (int jw = j; jw <= nw; jw += G) {
+                const int ka = max(wb + 32 * jw, klo), kz = min(wb + 32 * jw + 31, khi);
+                if (ka <= kz && window_maybe(g, o, d, ka, kz)) m |= 1u << jw;
+              }
+            }
+#pragma unroll
+            for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
+            if (now) {
+              wm = m;
+              need_mask = wm == 0u && wb + 1024 <= ke;
+              if (need_mask) wb += 1024;
             }
           }
+          if (__any_sync(kFull, todo == 0u && wm != 0u)) {
+            // the window's evaluated indices (bit i: index k0 + i): of this
+            // lane's ray (own), and of any ray of the frame (todo)
+            const bool now = todo == 0u && wm != 0u;
+            unsigned m = 0;
+            if (now) {
+              k0 = wb + 32 * (__ffs(wm) - 1);
+              if (alive) m = window_samples<G>(g, o, d, k0, klo, khi, j);
+              own = m;
+              wm &= wm - 1u;
+              need_mask = wm == 0u && wb + 1024 <= ke;
+              if (need_mask) wb += 1024;
+            }
 #pragma unroll
-          for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
-          if (now) {
-            wm = m;
-            need_mask = wm == 0u && wb + 1024 <= ke;
-            if (need_mask) wb += 1024;
+            for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
+            if (now) todo = m;
+            continue;
           }
+          if (!__any_sync(kFull, todo != 0u)) break;
         }
-        if (__any_sync(kFull, todo == 0u && wm != 0u)) {
-          // the window's evaluated indices (bit i: index k0 + i): of this
-          // lane's ray (own), and of any ray of the frame (todo)
-          const bool now = todo == 0u && wm != 0u;
-          unsigned m = 0;
-          if (now) {
-            k0 = wb + 32 * (__ffs(wm) - 1);
-            if (alive) m = window_samples<G>(g, o, d, k0, klo, khi, j);
-            own = m;
-            wm &= wm - 1u;
-            need_mask = wm == 0u && wb + 1024 <= ke;
-            if (need_mask) wb += 1024;
+        // G = 1: the frame's next index, for the rays evaluated there; else the
+        // ray's next G samples, one per lane
+        unsigned left = todo;
+        const unsigned had = todo;
+        if (G == 1) {
+          todo &= todo - 1u;
+        } else {
+#pragma unroll
+          for (int i = 0; i < G - 1; i++) {
+            if (i < j) left &= left - 1u;
+            todo &= todo - 1u;
           }
-#pragma unroll
-          for (int s = 1; s < kFrame; s <<= 1) m |= __shfl_xor_sync(kFull, m, s);
-          if (now) todo = m;
-          continue;
-        }
-        if (!__any_sync(kFull, todo != 0u)) break;
-      }
-      // G = 1: the frame's next index, for the rays evaluated there; else the
-      // ray's next G samples, one per lane
-      unsigned left = todo;
-      const unsigned had = todo;
-      if (G == 1) {
-        todo &= todo - 1u;
-      } else {
-#pragma unroll
-        for (int i = 0; i < G - 1; i++) {
-          if (i < j) left &= left - 1u;
           todo &= todo - 1u;
         }
-        todo &= todo - 1u;
-      }
-      const int bit = __ffs(left) - 1;
-      bool hit = alive && left != 0u && (G != 1 || ((own >> bit) & 1u));
-      float p[3] = {0.0f, 0.0f, 0.0f};
-      float2 zb = make_float2(0.0f, 0.0f);
-      if (hit) {
-        lattice_point(g, o, d, k0 + bit, p);
-        zb = __ldg(g.occ + occ_cell(g, p));
-      }
-      if (G == 1) {
+        const int bit = __ffs(left) - 1;
+        bool hit = alive && left != 0u && (G != 1 || ((own >> bit) & 1u));
+        float p[3] = {0.0f, 0.0f, 0.0f};
+        float2 zb = make_float2(0.0f, 0.0f);
         if (hit) {
-          float t[8], t0;
-          gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
-          SampleAct s;
-          activate(g, t, p[2], zb, s);
-          seen++;
-          if (!COUNT || !done) {
-            const float w = __fmul_rn(T.value(), s.ah);
-#pragma unroll
-            for (int c = 0; c < 4; c++) add_to2(F2[c], E2[c], w, s.x[2 * c], c < 3 ? s.x[2 * c + 1] : 0.0f);
-            T.pass(__fsub_rn(1.0f, s.ah));
-            done = T.value() < g.t_thr;
-          }
-          if (COUNT && !counted) {
-            t[0] = t0;
+          lattice_point(g, o, d, k0 + bit, p);
+          zb = __ldg(g.occ + occ_cell(g, p));
+        }
+        if (G == 1) {
+          if (hit) {
+            float t[8], t0;
+            gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
+            SampleAct s;
             activate(g, t, p[2], zb, s);
-            Tc.pass(__fsub_rn(1.0f, s.ah));
-            cnt = seen;
-            counted = Tc.value() < g.t_thr;
-            amb |= fabsf(Tc.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
+            seen++;
+            if (!COUNT || !done) {
+              const float w = __fmul_rn(T.value(), s.ah);
+#pragma unroll
+              for (int c = 0; c < 4; c++) add_to2(F2[c], E2[c], w, s.x[2 * c], c < 3 ? s.x[2 * c + 1] : 0.0f);
+              T.pass(__fsub_rn(1.0f, s.ah));
+              done = T.value() < g.t_thr;
+            }
+            if (COUNT && !counted) {
+              t[0] = t0;
+              activate(g, t, p[2], zb, s);
+              Tc.pass(__fsub_rn(1.0f, s.ah));
+              cnt = seen;
+              counted = Tc.value() < g.t_thr;
+              amb |= fabsf(Tc.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
+            }
+            alive = seen < g.n_max && !(done && (!COUNT || counted));
+            if (COUNT && !alive) kstop = k0 + bit;
           }
-          alive = seen < g.n_max && !(done && (!COUNT || counted));
-          if (COUNT && !alive) kstop = k0 + bit;
-        }
-        const unsigned am = __ballot_sync(kFull, alive);
-        if (((am >> base) & kFrameMask) == 0u) {
-          todo = wm = 0u;
-          need_mask = false;
-        }
-      } else {
-        hit = hit && seen + j < g.n_max;
-        SampleAct s;
-        s.ah = 0.0f;
-        float ahc = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 7; c++) s.x[c] = 0.0f;
-        if (hit) {
-          float t[8], t0;
-          gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
-          activate(g, t, p[2], zb, s);
-          if (COUNT) {
-            SampleAct sc;
-            t[0] = t0;
-            activate(g, t, p[2], zb, sc);
-            ahc = sc.ah;
+          const unsigned am = __ballot_sync(kFull, alive);
+          if (((am >> base) & kFrameMask) == 0u) {
+            todo = wm = 0u;
+            need_mask = false;
           }
-        }
-        if (!COUNT || __any_sync(kFull, !done)) {
-          // transmittance before each lane's sample, in lattice order
-          int last;
-          Through before = T, after;
-          chain<G>(before, after, s.ah, hit, j, base, g.t_thr, last);
-          const unsigned kept = hits_of<G>(hit && !done && j <= last, base);
-          const float w = __fmul_rn(before.value(), s.ah);
-          // lane j sums its channels, sample after sample
-          float v[8];
+        } else {
+          hit = hit && seen + j < g.n_max;
+          SampleAct s;
+          s.ah = 0.0f;
+          float ahc = 0.0f;
 #pragma unroll
-          for (int c = 0; c < 8; c++) v[c] = c < 7 ? s.x[c] : 0.0f;
-          transpose_lanes<G>(v, j);
-#pragma unroll
-          for (int i = 0; i < G; i++) {
-            const float wi = __shfl_sync(kFull, w, i, G);
-            if ((kept >> i) & 1u) {
-              if (G == 4) add_to2(F2[0], E2[0], wi, v[i], v[(4 + i) & 7]);
-              else add_to(F, E, wi, v[i]);
+          for (int c = 0; c < 7; c++) s.x[c] = 0.0f;
+          if (hit) {
+            float t[8], t0;
+            gather_features_eo<SPARSE, COUNT>(g, p, t, t0);
+            activate(g, t, p[2], zb, s);
+            if (COUNT) {
+              SampleAct sc;
+              t[0] = t0;
+              activate(g, t, p[2], zb, sc);
+              ahc = sc.ah;
             }
           }
-          const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
-          const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
-          if (!done) {
-            T.h = th;
-            T.l = tl;
+          if (!COUNT || __any_sync(kFull, !done)) {
+            // transmittance before each lane's sample, in lattice order
+            int last;
+            Through before = T, after;
+            chain<G>(before, after, s.ah, hit, j, base, g.t_thr, last);
+            const unsigned kept = hits_of<G>(hit && !done && j <= last, base);
+            const float w = __fmul_rn(before.value(), s.ah);
+            // lane j sums its channels, sample after sample
+            float v[8];
+#pragma unroll
+            for (int c = 0; c < 8; c++) v[c] = c < 7 ? s.x[c] : 0.0f;
+            transpose_lanes<G>(v, j);
+#pragma unroll
+            for (int i = 0; i < G; i++) {
+              const float wi = __shfl_sync(kFull, w, i, G);
+              if ((kept >> i) & 1u) {
+                if (G == 4) add_to2(F2[0], E2[0], wi, v[i], v[(4 + i) & 7]);
+                else add_to(F, E, wi, v[i]);
+              }
+            }
+            const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
+            const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
+            if (!done) {
+              T.h = th;
+              T.l = tl;
+            }
+            done = done || last < G;
           }
-          done = done || last < G;
-        }
-        if (COUNT && __any_sync(kFull, !counted)) {
-          int last;
-          Through before = Tc, after;
-          chain<G>(before, after, ahc, hit, j, base, g.t_thr, last);
-          const bool kept = hit && !counted && j <= last;
-          const int n = __popc(hits_of<G>(kept, base));
-          if (!counted) cnt = seen + n;
-          amb |= kept && fabsf(after.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
-          const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
-          const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
-          if (!counted) {
-            Tc.h = th;
-            Tc.l = tl;
+          if (COUNT && __any_sync(kFull, !counted)) {
+            int last;
+            Through before = Tc, after;
+            chain<G>(before, after, ahc, hit, j, base, g.t_thr, last);
+            const bool kept = hit && !counted && j <= last;
+            const int n = __popc(hits_of<G>(kept, base));
+            if (!counted) cnt = seen + n;
+            amb |= kept && fabsf(after.value() - g.t_thr) < g.t_thr * ambiguity(cnt);
+            const float th = __shfl_sync(kFull, after.h, min(last, G - 1), G);
+            const float tl = __shfl_sync(kFull, after.l, min(last, G - 1), G);
+            if (!counted) {
+              Tc.h = th;
+              Tc.l = tl;
+            }
+            counted = counted || last < G;
           }
-          counted = counted || last < G;
-        }
-        seen += __popc(hits_of<G>(hit, base));
-        if (seen >= g.n_max || (done && (!COUNT || counted))) {
-          if (COUNT && alive) kstop = k0 + 31 - __clz(had & ~todo);
-          alive = need_mask = false;
-          todo = wm = 0u;
+          seen += __popc(hits_of<G>(hit, base));
+          if (seen >= g.n_max || (done && (!COUNT || counted))) {
+            if (COUNT && alive) kstop = k0 + 31 - __clz(had & ~todo);
+            alive = need_mask = false;
+            todo = wm = 0u;
+          }
         }
       }
-    }
 
-    if (COUNT && G > 1) amb = hits_of<G>(amb, lane & ~(G - 1)) != 0u;
-    float out[3];
-    if (G == 1) {
-      if (valid) {
-        float yd[3] = {0.0f, 0.0f, 0.0f}, all[7];
+      if (COUNT && G > 1) amb = hits_of<G>(amb, lane & ~(G - 1)) != 0u;
+      float out[3];
+      if (G == 1) {
+        if (valid) {
+          float yd[3] = {0.0f, 0.0f, 0.0f}, all[7];
 #pragma unroll
-        for (int c = 0; c < 7; c++) all[c] = c & 1 ? F2[c / 2].y + E2[c / 2].y : F2[c / 2].x + E2[c / 2].x;
-        if (seen > 0) mlp_rays<1>(sW, all, d, 0, yd);
+          for (int c = 0; c < 7; c++) all[c] = c & 1 ? F2[c / 2].y + E2[c / 2].y : F2[c / 2].x + E2[c / 2].x;
+          if (seen > 0) mlp_rays<1>(sW, all, d, 0, yd);
 #pragma unroll
-        for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T.value(), g.bg[c], all[c] + yd[c]) : g.bg[c];
+          for (int c = 0; c < 3; c++) out[c] = seen > 0 ? fmaf(T.value(), g.bg[c], all[c] + yd[c]) : g.bg[c];
 #pragma unroll
-        for (int c = 0; c < 3; c++) a.rgb[3 * rid + c] = out[c];
-        if (COUNT && !amb) a.count[rid] = cnt;
-      }
-    } else if (half == 0) {
-      float y[3] = {0.0f, 0.0f, 0.0f};
-      const float Fj = G == 4 ? F2[0].x + E2[0].x : F + E;  // channel j
-      if (__any_sync(kFull, seen > 0)) {
-        float all[7];
+          for (int c = 0; c < 3; c++) a.rgb[3 * rid + c] = out[c];
+          if (COUNT && !amb) a.count[rid] = cnt;
+        }
+      } else if (half == 0) {
+        float y[3] = {0.0f, 0.0f, 0.0f};
+        const float Fj = G == 4 ? F2[0].x + E2[0].x : F + E;  // channel j
+        if (__any_sync(kFull, seen > 0)) {
+          float all[7];
 #pragma unroll
-        for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, c < G ? Fj : F2[0].y + E2[0].y, c % G, G);
-        mlp_rays<G>(sW, all, d, j, y);
-      }
-      if (valid && j < 3) {
-        a.rgb[3 * rid + j] = seen > 0 ? fmaf(T.value(), g.bg[j], Fj + y[0]) : g.bg[j];
-        if (COUNT && j == 0 && !amb) a.count[rid] = cnt;
-      }
-    }
-    if constexpr (!COUNT) {
-      break;
-    } else {
-      // does a ray of the bundle have to be counted again?
-      if (G == 1 ? !__any_sync(kFull, amb) : !__syncthreads_or(amb) && half == 0) break;
-      BundleCounts& bc = sCounts[G == 1 ? warp : 0];
-      const int more = cnt + 31 - seen;  // wanted beyond the samples it has seen
-      const int extra = samples_after<G>(g, o[0], o[1], o[2], d[0], d[1], d[2], kstop, khi,
-                                         valid && seen < g.n_max && kstop < khi ? more : 0, j);
-      if (j == 0) {
-        bc.count[slot] = cnt;
-        bc.samples[slot] = amb ? -1 : min(min(seen + extra, g.n_max), cnt + 31);
-      }
-      if (G == 8 && half == 0) continue;
-      if (G == 1) __syncwarp();
-      else __syncthreads();
-      if (G != 1 && warp != 0) break;
-      int x0 = 0, y0 = 0, place = 0;
-      long ray0 = ((long)sb * CamShape<G>::kRays) & ~31l;
-      const Cam* cam = nullptr;
-      if (a.use_cam) {
-        cam = &tile_camera<G>(a, sb, x0, y0, ray0);
-        if (G == 1) {
-          x0 += (warp & 1) * 8;
-          y0 += (warp >> 1) * 4;
+          for (int c = 0; c < 7; c++) all[c] = __shfl_sync(kFull, c < G ? Fj : F2[0].y + E2[0].y, c % G, G);
+          mlp_rays<G>(sW, all, d, j, y);
+        }
+        if (valid && j < 3) {
+          a.rgb[3 * rid + j] = seen > 0 ? fmaf(T.value(), g.bg[j], Fj + y[0]) : g.bg[j];
+          if (COUNT && j == 0 && !amb) a.count[rid] = cnt;
         }
       }
-#pragma unroll 1
-      for (unsigned again = __ballot_sync(kFull, bc.samples[lane] < 0), r = 0; r < 32 && again >> r; r++) {
-        if (!((again >> r) & 1u)) {
-          place = next_place(place, bc.count[r], bc.samples[r]);
-        } else {
-          // (a ray of the other half is counted for its place only)
-          float ro[3], rd[3];
-          bool own = true;
-          long id = ray0 + r;
-          if (a.use_cam) {
-            const int px = (x0 & ~7) + (r & 7), py = y0 + (r >> 3);
-            own = G != 8 || ((px ^ x0) & 4) == 0;
-            id = ray0 + (long)py * cam->width + px;
-            camera_ray(*cam, px, py, ro, rd);
-          } else {
-            own = G != 8 || (r >> 4) == (sb & 1u);
-            load_ray(a.rays + 6 * id, ro, rd);
-          }
-          const int n = count_in_queue<FT, SPARSE>(g, ro, rd, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0], lane, place);
-          if (own && lane == 0) a.count[id] = n;
+      if constexpr (!COUNT) {
+        break;
+      } else {
+        // does a ray of the bundle have to be counted again?
+        if (G == 1 ? !__any_sync(kFull, amb) : !__syncthreads_or(amb) && half == 0) break;
+        BundleCounts& bc = sCounts[G == 1 ? warp : 0];
+        const int more = cnt + 31 - seen;  // wanted beyond the samples it has seen
+        const int extra = samples_after<G>(g, o[0], o[1], o[2], d[0], d[1], d[2], kstop, khi,
+                                           valid && seen < g.n_max && kstop < khi ? more : 0, j);
+        if (j == 0) {
+          bc.count[slot] = cnt;
+          bc.samples[slot] = amb ? -1 : min(min(seen + extra, g.n_max), cnt + 31);
         }
+        // (narrow images' super-tiles hold whole bundles)
+        if (G == 8 && half == 0 && !(a.use_cam && whole_bundles<G>(a, sb))) continue;
+        if (G == 1) __syncwarp();
+        else __syncthreads();
+        if (G == 1 || warp == 0) count_again<FT, SPARSE, G>(g, a, sb, warp, bc, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0]);
+        break;
       }
-      break;
-    }
     }
     __syncthreads();
   }
@@ -794,9 +880,15 @@ int list_lanes(const omerf_scene* s, long n) {
   return s->desc.feat_dtype == OMERF_F32 && n < (1 << 14) ? 8 : 0;
 }
 
-void cam_super(int lanes, int& w, int& h) {
-  w = lanes == 0 ? 16 : (lanes == 1 ? CamShape<1>::kW : (lanes == 4 ? CamShape<4>::kW : CamShape<8>::kW));
-  h = lanes == 0 ? 16 : (lanes == 1 ? CamShape<1>::kH : (lanes == 4 ? CamShape<4>::kH : CamShape<8>::kH));
+void cam_super(int lanes, int width, int height, int& lw, int& w, int& h) {
+  lw = -1;
+  if (lanes == 0) {
+    w = h = 16;
+    return;
+  }
+  if (width <= (lanes == 8 ? 2 : 4)) lw = width < 3 ? width - 1 : 2;
+  else if (height <= 2) lw = (lanes == 8 ? 5 : 6) - height;
+  super_size(lanes, lw, w, h);
 }
 
 cudaError_t launch_render_cam(const omerf_scene* s, const FwdArgs& a, int lanes, cudaStream_t stream) {

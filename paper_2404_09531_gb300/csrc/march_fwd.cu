@@ -257,15 +257,14 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
     a.use_cam = 1;
     int sw, sh;
     lanes = cam_lanes(s, n);
-    cam_super(lanes, sw, sh);
+    cam_super(lanes, cam->width, cam->height, a.lw, sw, sh);
     a.super_x = (cam->width + sw - 1) / sw;
     a.n_super = (long)a.super_x * ((cam->height + sh - 1) / sh);
   } else {
     a.use_cam = 0;
     lanes = train ? 0 : list_lanes(s, n);
-    int sw = 32, sh = 1;
-    if (lanes > 0) cam_super(lanes, sw, sh);
-    a.n_super = (n + sw * sh - 1) / (sw * sh);
+    const int per = lanes > 0 ? 16 : 32;  // rays of a CTA with 8 lanes per ray, or of a warp
+    a.n_super = (n + per - 1) / per;
   }
   a.rays = rays;
   a.n = n;

@@ -109,7 +109,7 @@ __device__ __forceinline__ void march_bundle(const Geo& g, int lane, const float
 
 struct FwdArgs {
   Cam cam;
-  int use_cam, super_x;
+  int use_cam, super_x, lw;  // lw: the super-tiles' form (march_cam.cu)
   const float* rays;
   long n, n_super;
   float* rgb;

@@ -780,16 +780,15 @@ omerf_status omerf_render_cameras(const omerf_scene* s, const omerf_camera* cams
     long supers = 0, rays = 0;
     for (int c = 0; c < m; c++) rays += (long)cams[c0 + c].width * cams[c0 + c].height;
     const int lanes = cam_lanes(s, rays);
-    int sw, sh;
-    cam_super(lanes, sw, sh);
     rays = 0;
     for (int c = 0; c < m; c++) {
       const omerf_camera& k = cams[c0 + c];
+      int sw, sh;
       rec[c].cam = to_cam(&k);
+      cam_super(lanes, k.width, k.height, rec[c].lw, sw, sh);
       rec[c].super_x = (k.width + sw - 1) / sw;
       rec[c].super_start = supers;
       rec[c].ray_start = rays;
-      rec[c].pad = 0;
       supers += (long)rec[c].super_x * ((k.height + sh - 1) / sh);
       rays += (long)k.width * k.height;
     }

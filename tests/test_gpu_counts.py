@@ -126,3 +126,29 @@ def test_counts_of_opaque_samples_in_ramps():
             _, queue = om.render(scene, rays=rays)
             _, short = om.render(scene, rays=rays[:8192].contiguous())
             assert torch.equal(short, queue[:8192])
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (1, 701), (2, 301), (3, 99), (4, 97), (701, 1), (301, 2), (99, 3), (2, 2), (6, 1),
+                                 (5, 2)])
+def test_narrow_images(w, h):
+    """Images of a few columns or rows have super-tiles of their own: the same
+    pixels in every form, and the counts of the 8 x 4 tiles in the queue (those
+    that training saves), a good part of them decided by rounding."""
+    scene = gpu_scene(_fog(0.004, holes=True), t_thr=0.3)
+    cam = _camera(w, h)
+    if w > 8 * h:
+        cam["fx"] = cam["fy"] = np.float32(w)
+    tiled, back = _tiles(oracle.camera_rays(cam), w, h)
+    _, saved, _ = om.train_fwd(scene, tiled, torch.zeros(tiled.shape[0], 3, device="cuda"))
+    want = saved.view(-1, 20)[:, 8].contiguous().view(torch.int32)[back]
+    rgb, cnt = om.render(scene, camera=cam)
+    assert torch.equal(cnt, want)
+    assert torch.equal(om.render(scene, camera=cam, want_count=False)[0], rgb)
+    for fill in (_camera(512, 300), _camera(1024, 1024)):
+        g_rgb, g = om.render_cameras(scene, [cam, fill, cam])
+        assert torch.equal(g[: w * h], want) and torch.equal(g_rgb[: w * h], rgb)
+        assert torch.equal(g[-w * h:], want) and torch.equal(g_rgb[-w * h:], rgb)
+        p_rgb, _ = om.render_cameras(scene, [cam, fill], want_count=False)
+        assert torch.equal(p_rgb[: w * h], rgb)
+    rays = torch.as_tensor(oracle.camera_rays(cam)).cuda()
+    assert torch.equal(om.render(scene, rays=rays[:4096].contiguous(), want_count=False)[0], rgb[:4096])
