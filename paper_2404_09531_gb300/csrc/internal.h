@@ -79,7 +79,7 @@ cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int 
 
 // Lanes that march one ray of a camera render of n rays (0: the packed
 // queue of march_fwd.cu), and form and pixels of the super-tile a CTA takes.
-int cam_lanes(const omerf_scene* s, long n);
+int cam_lanes(const omerf_scene* s, long n, bool count);
 int list_lanes(const omerf_scene* s, long n);  // the same for a ray list (kRays rays per CTA)
 void cam_super(int lanes, int width, int height, int& lw, int& w, int& h);
 

@@ -860,15 +860,27 @@ static cudaError_t launch_cam_group(const omerf_scene* s, const FwdArgs& a, cuda
                            : launch_cam_variant<float, false, G, COUNT>(s, a, stream);
 }
 
-// The lines lie where the measured times cross (us with 8 / 4 / 1 lanes; city
-// unless said): 57,600 rays 208 / 267 / 549, 129,600 rays 320 / 331 / 711,
-// 230,400 rays 490 / 455 / 833, 518,400 rays 1003 / 852 / 1027, 921,600 rays
-// 1708 / 1419 / 1387, 1,048,576 rays (field) 848 / 632 / 469.  A BF16
-// scene keeps the packed queue: its deferred MLP rounds F to bfloat16, so sums
-// in another order would move pixels by a step of that rounding.
-int cam_lanes(const omerf_scene* s, long n) {
+// The lines lie where the measured times cross.  In a box of many lattice
+// steps' height rays hold more samples and differ more, so that a warp of whole
+// rays waits longer for its last one and needs a larger image; and the counting
+// form of one lane per ray, with fewer warps per SM, needs a smaller one.
+// us with 8 / 4 / 1 lanes, means of three scenes:
+//   city (256 steps)  129,600 rays 285 / 301 / 696, 176,400 356 / 356 / 770,
+//     518,400 920 / 834 / 966, 705,600 1233 / 1105 / 1153, 921,600 1586 / 1409 /
+//     1370; with counts 176,400 426 / 441 / 706, 360,000 808 / 739 / 809, 518,400
+//     1130 / 1005 / 979
+//   field (64 steps)  65,536 72 / 73 / 115, 102,400 99 / 92 / 146, 262,144 216 /
+//     183 / 193, 409,600 323 / 268 / 233; with counts 65,536 89 / 89 / 116,
+//     147,456 170 / 144 / 177, 200,704 222 / 182 / 186, 262,144 283 / 226 / 191
+// (the city's first line is within 6 % of the better form from 2^17 to 2^18).
+// A BF16 scene keeps the packed queue: its deferred MLP rounds F to bfloat16, so
+// sums in another order would move pixels by a step of that rounding.
+int cam_lanes(const omerf_scene* s, long n, bool count) {
   if (s->desc.feat_dtype != OMERF_F32) return 0;
-  return n < (1 << 17) ? 8 : (n < (3 << 18) ? 4 : 1);
+  const bool tall = s->geo.hi[2] - s->geo.lo[2] > 128.0f * s->geo.step;
+  const long eight = tall ? 1 << 17 : 5 << 14;
+  const long four = tall ? (count ? 7 << 16 : 3 << 18) : (count ? 3 << 16 : 5 << 16);
+  return n < eight ? 8 : (n < four ? 4 : 1);
 }
 
 // Rays of a list may lie anywhere: rays of different lengths share a warp, and

@@ -256,7 +256,7 @@ cudaError_t launch_march_fwd(const omerf_scene* s, const Cam* cam, const float* 
     a.cam = *cam;
     a.use_cam = 1;
     int sw, sh;
-    lanes = cam_lanes(s, n);
+    lanes = cam_lanes(s, n, count != nullptr);
     cam_super(lanes, cam->width, cam->height, a.lw, sw, sh);
     a.super_x = (cam->width + sw - 1) / sw;
     a.n_super = (long)a.super_x * ((cam->height + sh - 1) / sh);

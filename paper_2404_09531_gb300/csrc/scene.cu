@@ -779,7 +779,7 @@ omerf_status omerf_render_cameras(const omerf_scene* s, const omerf_camera* cams
     CamRec rec[kMaxCams];
     long supers = 0, rays = 0;
     for (int c = 0; c < m; c++) rays += (long)cams[c0 + c].width * cams[c0 + c].height;
-    const int lanes = cam_lanes(s, rays);
+    const int lanes = cam_lanes(s, rays, cd != nullptr);
     rays = 0;
     for (int c = 0; c < m; c++) {
       const omerf_camera& k = cams[c0 + c];
