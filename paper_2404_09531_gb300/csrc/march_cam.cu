@@ -885,11 +885,15 @@ int cam_lanes(const omerf_scene* s, long n, bool count) {
 
 // Rays of a list may lie anywhere: rays of different lengths share a warp, and
 // the queue, which packs samples whatever their ray, keeps its lanes busy.  Few
-// rays leave the chip idle, and there 8 lanes per ray shorten the chain (us
-// with the queue / 8 lanes, random city rays with counts: 3,001 rays 253 /
-// 180, 10,007 rays 256 / 176, 30,011 rays 259 / 276, 100,003 rays 319 / 693).
+// rays leave the chip idle, and there 8 lanes per ray shorten the chain, but a
+// handful of rays goes through the queue with all 32 lanes on one ray.  us with
+// the queue / 8 lanes, random city rays with counts: 1 ray 18 / 25, 6 rays 39 /
+// 40, 12 rays 63 / 50, 8,192 rays 220 / 105, 16,383 rays 226 / 177, 30,000 rays
+// 232 / 229, 40,000 rays 236 / 274; field: 6 rays 22 / 26, 12 rays 31 / 27, 16,383
+// rays 86 / 72, 24,576 rays 87 / 80, 30,000 rays 87 / 95.  The upper line lies
+// below all crossings.
 int list_lanes(const omerf_scene* s, long n) {
-  return s->desc.feat_dtype == OMERF_F32 && n < (1 << 14) ? 8 : 0;
+  return s->desc.feat_dtype == OMERF_F32 && n > 6 && n < (1 << 14) ? 8 : 0;
 }
 
 void cam_super(int lanes, int width, int height, int& lw, int& w, int& h) {

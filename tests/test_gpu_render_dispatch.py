@@ -1,13 +1,14 @@
 """Renders on both sides of every line of the dispatch (lanes per ray by the rays
-of the launch, the box's height in lattice steps and whether counts are wanted):
-the same pixels and counts."""
+of the launch, the box's height in lattice steps and whether counts are wanted;
+short lists): the same pixels and counts."""
 import numpy as np
 import pytest
 import torch
 
+import oracle
 import synth
 import paper_2404_09531_gb300 as om
-from _util import brick_inputs, gpu_scene
+from _util import brick_inputs, compare_render, gpu_scene, oracle_scene_for
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +46,17 @@ def test_launches_beside_the_lines(cfg, count):
             assert torch.equal(rgb[:n], want)
             if count:
                 assert torch.equal(cnt[:n], want_cnt)
+
+
+@pytest.mark.parametrize("cfg", [1, 2])
+@pytest.mark.parametrize("n", [1, 5, 6, 7, 8])
+def test_a_handful_of_listed_rays(cfg, n):
+    sc, table, pool, scene = _scene(cfg)
+    rays = synth.make_train_batch(cfg, 4096, K=1)["rays"]
+    for at in (0, 1000, 2048):
+        part = np.ascontiguousarray(rays[at:at + n])
+        rgb, cnt = om.render(scene, rays=part)
+        assert torch.equal(om.render(scene, rays=part, want_count=False)[0], rgb)
+        ref = oracle.render(oracle_scene_for(sc, table, pool), part)
+        if (ref["ambiguous"] == 0).all():
+            compare_render(rgb.cpu().numpy(), cnt.cpu().numpy(), ref, what=f"config {cfg}, {n} rays")
