@@ -417,7 +417,7 @@ __device__ __noinline__ int samples_after(const Geo& g, float o0, float o1, floa
 
 // Count a ray (the same one in every lane) as the queue does from `place`, and
 // move `place` on.
-template <class FT, bool SPARSE>
+template <bool SPARSE>
 __device__ __forceinline__ int count_in_queue(const Geo& g, const float o[3], const float d[3], float4* sa, float* sb,
                                               int lane, int& place) {
   int klo = 0, khi = -1, count = 0, nq = place, first = place, taken = 0;
@@ -433,7 +433,7 @@ __device__ __forceinline__ int count_in_queue(const Geo& g, const float o[3], co
       const float4 q = sa[lane];
       const float p[3] = {q.x, q.y, q.z};
       float t[8];
-      gather_features<FT, SPARSE>(g, p, t);
+      gather_features<float, SPARSE>(g, p, t);
       activate(g, t, p[2], make_float2(q.w, sb[lane]), s);
     }
     const float Tn = T * seg_prod_scan(__fsub_rn(1.0f, s.ah), lane, first);
@@ -486,7 +486,7 @@ __device__ __noinline__ bool whole_bundles(const FwdArgs& a, unsigned sb) {
 
 // Count the ambiguous rays of a warp's (G = 1) or a CTA's bundles, and write
 // their counts (a call of its own, so that the march keeps its registers).
-template <class FT, bool SPARSE, int G>
+template <bool SPARSE, int G>
 __device__ __noinline__ void count_again(const Geo& g, const FwdArgs& a, unsigned sb, int warp, const BundleCounts& bc,
                                          float4* qa, float* qb) {
   const int lane = threadIdx.x & 31;
@@ -526,7 +526,7 @@ __device__ __noinline__ void count_again(const Geo& g, const FwdArgs& a, unsigne
       own = G != 8 || (r >> 4) == (sb & 1u);
       load_ray(a.rays + 6 * id, o, d);
     }
-    const int n = count_in_queue<FT, SPARSE>(g, o, d, qa, qb, lane, place);
+    const int n = count_in_queue<SPARSE>(g, o, d, qa, qb, lane, place);
     if (own && lane == 0) a.count[id] = n;
   }
 }
@@ -535,7 +535,7 @@ __device__ __noinline__ void count_again(const Geo& g, const FwdArgs& a, unsigne
 // counts (a second density sum in registers) with 4, 5 2.60, 2.94 ms; 641x361
 // with 5, 6 for G = 4 417, 434 us; 320x180 with 6, 7 for G = 8 242, 208 us;
 // 10,007 listed rays with counts with 4, 5 for G = 8 180, 144 us.
-template <class FT, bool SPARSE, int G, bool COUNT>
+template <bool SPARSE, int G, bool COUNT>
 __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 : 5) : (G == 8 ? 7 : 5))
     march_cam_kernel(const __grid_constant__ Geo g, const __grid_constant__ FwdArgs a) {
   constexpr int kFrame = G == 8 ? 8 : 4;           // lanes that share a lattice frame
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
         if (G == 8 && half == 0 && !(a.use_cam && whole_bundles<G>(a, sb))) continue;
         if (G == 1) __syncwarp();
         else __syncthreads();
-        if (G == 1 || warp == 0) count_again<FT, SPARSE, G>(g, a, sb, warp, bc, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0]);
+        if (G == 1 || warp == 0) count_again<SPARSE, G>(g, a, sb, warp, bc, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0]);
         break;
       }
     }
@@ -836,9 +836,9 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
   }
 }
 
-template <class FT, bool SPARSE, int G, bool COUNT>
+template <bool SPARSE, int G, bool COUNT>
 static cudaError_t launch_cam_variant(const omerf_scene* s, const FwdArgs& a, cudaStream_t stream) {
-  auto kern = march_cam_kernel<FT, SPARSE, G, COUNT>;
+  auto kern = march_cam_kernel<SPARSE, G, COUNT>;
   constexpr int threads = 32 * CamShape<G>::kWarps;
   static std::atomic<int> blocks[64];  // per device: resident CTAs of this variant
   const int dev = s->device & 63;
@@ -856,8 +856,8 @@ static cudaError_t launch_cam_variant(const omerf_scene* s, const FwdArgs& a, cu
 
 template <int G, bool COUNT>
 static cudaError_t launch_cam_group(const omerf_scene* s, const FwdArgs& a, cudaStream_t stream) {
-  return s->desc.brick > 0 ? launch_cam_variant<float, true, G, COUNT>(s, a, stream)
-                           : launch_cam_variant<float, false, G, COUNT>(s, a, stream);
+  return s->desc.brick > 0 ? launch_cam_variant<true, G, COUNT>(s, a, stream)
+                           : launch_cam_variant<false, G, COUNT>(s, a, stream);
 }
 
 // The lines lie where the measured times cross.  In a box of many lattice

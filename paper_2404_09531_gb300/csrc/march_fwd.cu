@@ -47,16 +47,17 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
   WarpMarch<kMMA>& ws = sMarch[threadIdx.x >> 5];
   float l_rgb = 0.0f, l_smooth = 0.0f;
 
-  // A camera: the CTA takes super-tiles of 2 x 4 tiles of 8 x 4 pixels (16 x
-  // 16 pixels), so that its 8 warps march neighbouring rays together and share
-  // L1 lines.  A list: every warp takes its next 32 consecutive rays on its
-  // own, without waiting for the CTA's slowest bundle (the rays of a training
-  // batch lie anywhere).  Without a counter there is one unit per CTA or warp.
+  // A camera (of a BF16 scene; FP32 ones are marched by march_cam.cu): the CTA
+  // takes super-tiles of 2 x 4 tiles of 8 x 4 pixels (16 x 16 pixels), so that
+  // its 8 warps march neighbouring rays together and share L1 lines.  A list:
+  // every warp takes its next 32 consecutive rays on its own, without waiting
+  // for the CTA's slowest bundle (the rays of a training batch lie anywhere).
+  // Without a counter there is one unit per CTA or warp.
   __shared__ unsigned sWork;
   const int warp = threadIdx.x >> 5;
   for (bool first = true;; first = false) {
     unsigned sb;
-    if (a.use_cam) {
+    if (kMMA && a.use_cam) {
       if (threadIdx.x == 0)
         sWork = a.counter ? atomicAdd(a.counter, 1u) : (first ? blockIdx.x : (unsigned)a.n_super);
       __syncthreads();
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
     long rid;
     bool valid;
     float o[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 1.0f};
-    if (a.n_cams > 0) {
+    if (kMMA && a.n_cams > 0) {
       int c = 0;
       while (c + 1 < a.n_cams && (long long)sb >= a.cams[c + 1].super_start) c++;
       const CamRec& cr = a.cams[c];
@@ -85,7 +86,7 @@ __global__ void __launch_bounds__(kThreads, OMERF_FWD_MINB) march_fwd_kernel(con
       valid = px < cr.cam.width && py < cr.cam.height;
       rid = (long)cr.ray_start + (long)py * cr.cam.width + px;
       if (valid) camera_ray(cr.cam, px, py, o, d);
-    } else if (a.use_cam) {
+    } else if (kMMA && a.use_cam) {
       const int sx = (int)(sb % (unsigned)a.super_x), sy = (int)(sb / (unsigned)a.super_x);
       const int tx = 2 * sx + (warp & 1), ty = 4 * sy + (warp >> 1);
       const int px = tx * 8 + (lane & 7), py = ty * 4 + (lane >> 3);
@@ -312,11 +313,9 @@ cudaError_t launch_march_fwd_cams(const omerf_scene* s, const CamRec* cams, int 
   a.count = count;
   if (a.n_super == 0) return cudaSuccess;
   if (lanes > 0) return launch_render_cam(s, a, lanes, stream);
-  const bool bf16 = s->desc.feat_dtype == OMERF_BF16;
-  const bool sparse = s->desc.brick > 0;
-  if (bf16) return sparse ? launch_variant<__nv_bfloat16, true, false>(s, a, stream)
-                          : launch_variant<__nv_bfloat16, false, false>(s, a, stream);
-  return sparse ? launch_variant<float, true, false>(s, a, stream) : launch_variant<float, false, false>(s, a, stream);
+  // (a BF16 scene)
+  return s->desc.brick > 0 ? launch_variant<__nv_bfloat16, true, false>(s, a, stream)
+                           : launch_variant<__nv_bfloat16, false, false>(s, a, stream);
 }
 
 }  // namespace omerf
