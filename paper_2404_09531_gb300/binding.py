@@ -122,12 +122,15 @@ def _check(status: int, what: str):
         raise OmerfError(f"{what} failed with status {status}: {msg.decode() if msg else ''}")
 
 
+# The current stream of a device without a Stream object around it (about 5 us of
+# every call); not a public name of torch, so the public way remains beside it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
     if stream is None:
-        if torch.cuda.is_initialized():
-            # the current device's current stream, without building a Stream object
-            # around it (about 5 us of every call)
-            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
