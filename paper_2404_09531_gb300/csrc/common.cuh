@@ -281,8 +281,9 @@ struct Texel<__nv_bfloat16> {
 
 // t += w v over the 8 channels of a texel, two channels per packed FP32 FMA
 // (sm_100+; each half is one fused multiply-add rounded to nearest, exactly
-// as fmaf).  Used where the march is issue-bound (BF16 features); with FP32
-// features the scalar form keeps fewer registers live.
+// as fmaf).  Used by the queue where it is issue-bound (BF16 features; with FP32
+// features its scalar form keeps fewer registers live) and by the camera forms
+// (gather_features_eo).
 __device__ __forceinline__ void fma8x2(float2 t[4], float w, const float v[8]) {
   const float2 ww = make_float2(w, w);
 #pragma unroll

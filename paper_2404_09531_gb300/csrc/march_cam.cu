@@ -22,11 +22,11 @@
 // the other in the same order, so a pixel does not depend on G, nor on
 // whether counts are wanted.
 //
-// Measured on a GB300, 512 x 512 x 32 city, against the packed queue:
-// 8 x 1920x1080 29.4 -> 20.3 ms (L1 pipe 83 % busy, 1.8 G instead of 2.7 G
-// instructions per frame), 1920x1080 3.80 -> 2.55 ms (G = 4: 3.01), 640x360
-// 0.83 -> 0.46 ms (G = 8: 0.49, G = 1: 0.83), 64x64 of the 64 x 64 x 16 field
-// 0.155 -> 0.053 ms (G = 4: 0.064).
+// Measured on a GB300, 512 x 512 x 32 city, against the packed queue: 8 x
+// 1920x1080 29.4 -> 19.4 ms (L1 pipe 81 % busy, 1.9 G instead of 2.7 G
+// instructions per frame), 1920x1080 3.75 -> 2.53 ms, 640x360 0.83 -> 0.43 ms (G =
+// 8: 0.45, G = 1: 0.78), 64x64 of the 64 x 64 x 16 field with counts 0.113 ->
+// 0.030 ms.
 //
 // Sample counts are those of the packed queue, which training and long ray
 // lists use, also where rounding decides them.  The two forms multiply a
@@ -41,8 +41,8 @@
 namespace omerf {
 
 // Warps per CTA and the pixels of its super-tile (whole or half 8 x 4 tiles).
-// CTAs of 4 warps wait less for their slowest tile than CTAs of 8 (2.96
-// against 3.10 ms per 1080p frame; 2 warps 3.05).
+// CTAs of 4 warps wait less for their slowest tile than CTAs of 8 (an earlier
+// state of the kernel: 2.96 against 3.10 ms per 1080p frame; 2 warps 3.05).
 template <int G>
 struct CamShape;
 template <>
@@ -275,7 +275,8 @@ __device__ __forceinline__ void transpose_lanes(float v[8], int j) {
 // after the other, where the packed queue's lane scans round a sample's
 // contribution about five times whatever the ray's length, and a plain sum
 // in order would be coarser (pixels of rays of 700 samples 3.7e-7 off 64-bit
-// ones instead of 1.8e-7, root mean square; with the compensation 1.6e-7.  It costs a 1080p frame 2 %).
+// ones instead of 1.8e-7, root mean square; with the compensation 1.6e-7; it
+// costs a 1080p frame 2 % and small images of few samples up to 5 %).
 //
 // Transmittance T = h + l, the rounding errors of h's products carried along.
 struct Through {
@@ -320,6 +321,7 @@ __device__ __forceinline__ void chain(Through& T, Through& after, float ah, bool
   const unsigned below = hits_of<G>(hit && after.value() < thr, base);
   last = below ? __ffs(below) - 1 : G;
 }
+
 // The camera of super-tile sb, its form (see SubTile), pixel origin and first ray.
 template <int G>
 __device__ __forceinline__ const Cam& tile_camera(const FwdArgs& a, unsigned sb, int& lw, int& x0, int& y0,
@@ -816,7 +818,8 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
       } else {
         // does a ray of the bundle have to be counted again?
         if (G == 1 ? !__any_sync(kFull, amb) : !__syncthreads_or(amb) && half == 0) break;
-        BundleCounts& bc = sCounts[G == 1 ? warp : 0];
+        const int home = G == 1 ? warp : 0;  // the warp that replays, and its places
+        BundleCounts& bc = sCounts[home];
         const int more = cnt + 31 - seen;  // wanted beyond the samples it has seen
         const int extra = samples_after<G>(g, o[0], o[1], o[2], d[0], d[1], d[2], kstop, khi,
                                            valid && seen < g.n_max && kstop < khi ? more : 0, j);
@@ -828,7 +831,7 @@ __global__ void __launch_bounds__(32 * CamShape<G>::kWarps, COUNT ? (G == 1 ? 4 
         if (G == 8 && half == 0 && !(a.use_cam && whole_bundles<G>(a, sb))) continue;
         if (G == 1) __syncwarp();
         else __syncthreads();
-        if (G == 1 || warp == 0) count_again<SPARSE, G>(g, a, sb, warp, bc, sQa[G == 1 ? warp : 0], sQb[G == 1 ? warp : 0]);
+        if (warp == home) count_again<SPARSE, G>(g, a, sb, warp, bc, sQa[home], sQb[home]);
         break;
       }
     }

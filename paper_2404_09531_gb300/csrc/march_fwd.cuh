@@ -17,11 +17,14 @@ struct MarchState {
   float T[32];       // per-ray transmittance so far
   int cnt[32];       // per-ray evaluated samples
 };
-// With the tensor-core MLP the whole march state doubles as the MLP staging
-// area: the epilogue copies each ray's F, T and count to registers before it
-// stages the MLP rows, and the next bundle starts after a CTA barrier.  The
-// smaller per-warp footprint lets the BF16 render take a smaller
-// shared-memory carveout, leaving more of the SM's SRAM to L1.
+// With the tensor-core MLP the whole march state doubles as the warp's MLP
+// staging area.  Two warp barriers separate the uses: the one after each ray's
+// F, T and count are copied to registers, before the MLP rows are staged, and
+// the one that ends mlp_bf16_warp, after the outputs are read and before the
+// next bundle's state is written (a warp takes its next bundle of a list on its
+// own: there is no CTA barrier in between).  The smaller per-warp footprint lets
+// the BF16 render take a smaller shared-memory carveout, leaving more of the
+// SM's SRAM to L1.
 template <bool MMA>
 struct WarpMarch {
   MarchState s;

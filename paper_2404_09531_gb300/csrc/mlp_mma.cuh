@@ -173,7 +173,7 @@ __device__ __forceinline__ void mlp_bf16_warp(const MlpFrags& f, MlpStage& st, i
   __syncwarp();
 #pragma unroll
   for (int j = 0; j < 3; j++) y[j] = sigmoidf_(st.Y[lane][j]);
-  __syncwarp();
+  __syncwarp();  // required: the caller may reuse the staging memory at once (WarpMarch<true>)
 }
 
 }  // namespace omerf

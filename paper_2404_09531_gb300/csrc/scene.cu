@@ -34,8 +34,9 @@ unsigned* next_counter(const omerf_scene* s, cudaStream_t stream) {
 // ---------------------------------------------------------------------------
 // occupancy hull: min z_min and max z_max over the non-empty cells
 // ---------------------------------------------------------------------------
-// One block (no second pass, no atomics): the loads of eight rounds are in
-// flight together (65,536 cells 10.0 us, 13.0 us one round at a time).
+// One block (no second pass, no atomics) over the cells of the coarse grid; the
+// loads of eight rounds are in flight together, for grids as fine as the
+// occupancy plane (65,536 cells 10.0 us, 13.0 us one round at a time).
 static __global__ void __launch_bounds__(1024) hull_kernel(const float2* __restrict__ occ, long cells,
                                                            float* __restrict__ hull) {
   __shared__ float slo[32], shi[32];
